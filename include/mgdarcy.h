@@ -90,8 +90,16 @@ typedef struct {
                            rounding).  -1: automatic (the largest j < J whose
                            matrix fits 2.5 GiB in the working precision),
                            0: never, j >= 1: level j.                          */
-  int pass_kernel;      /* kernel of the colour passes of the smoother (same
-                           update up to rounding): 1: one warp per patch
+  int pass_kernel;      /* kernel of the smoother (same update up to rounding).
+                           With 0 (default), 4 and 5 a smoothing step runs as
+                           line sweeps where the level's strips fit the shared
+                           memory: the three to five consecutive colour passes
+                           that differ in the x digit of the colour are one
+                           launch, a cluster of blocks per line of vertices (not
+                           with the additive variant, boundary_patches, a block
+                           limit, nor degree 2 in FP64).  The other values, and
+                           these where line sweeps do not apply, take one
+                           launch per colour pass: 1: one warp per patch
                            (persistent), 2: one thread block per patch,
                            3: persistent thread blocks, one patch at a time,
                            0 (default) or 4: per level, the fastest of the
@@ -99,10 +107,10 @@ typedef struct {
                            symmetric smoothing steps as a CUDA graph, see
                            mg_time_passes; cached per level shape, precision,
                            right-hand sides, problems of a batch group,
-                           smoother options and device; a level whose timed
-                           choice differs from the rule of 5 keeps it only if
-                           the whole V-cycle is faster with it, finest level
-                           first, mg_setup only), 5: a fixed rule
+                           smoother options and device; a level without line
+                           sweeps whose timed choice differs from the rule of 5
+                           keeps it only if the whole V-cycle is faster with it,
+                           finest level first, mg_setup only), 5: a fixed rule
                            (block kernel where the largest colour holds at
                            most 10,000 inverse entries per SM or four or more
                            right-hand sides share the inverses, else warp);
@@ -229,7 +237,8 @@ mg_status mg_set_wait_limit(mg_handle* h, double seconds);
  * concurrent work.  The kernels walk every patch of a colour whatever the
  * grid, and each patch's arithmetic does not depend on which block takes it,
  * so results are bit-identical for any cap (the test of one block walking a
- * whole colour relies on it).  Re-captures the V-cycle graph on its next use;
+ * whole colour relies on it).  With a cap the handle smooths by colour passes
+ * even where it would take line sweeps (mg_problem.pass_kernel).  Re-captures the V-cycle graph on its next use;
  * synchronises the stream. */
 mg_status mg_set_block_limit(mg_handle* h, int blocks);
 
@@ -425,7 +434,8 @@ mg_status mg_patch_nnz(const mg_handle* h, int level, int64_t* nnz);
 
 /* Average time in microseconds of one colour pass (Sec. 3.3) of `level`
  * (>= 1) with colour-pass kernel `kernel` (1 warp per patch, 2 block per
- * patch, 3 persistent blocks; 0: the level's own, see mg_level_pass_kernel):
+ * patch, 3 persistent blocks; 0: as the handle smooths this level, by line
+ * sweeps where they apply, else by the kernel of mg_level_pass_kernel):
  * two symmetric smoothing steps captured as a CUDA graph, replayed five times
  * between CUDA events after one untimed replay, so that the passes run back
  * to back as inside the V-cycle.  Overwrites the handle's level vectors of
@@ -453,7 +463,8 @@ mg_status mg_measure_fma_peak(int kind, double* tflops, void* cuda_stream);
  * and frees a small device buffer; synchronises the stream. */
 mg_status mg_measure_sync_cost(int kind, int blocks, double* us_per_step, void* cuda_stream);
 
-/* Colour-pass kernel chosen for `level` (1 <= level <= J) at setup, see
+/* Colour-pass kernel chosen for `level` (1 <= level <= J) at setup (what
+ * mg_colour_pass runs, and smoothing where line sweeps do not apply), see
  * mg_problem.pass_kernel: *kernel = 1 (warp per patch), 2 (block per patch)
  * or 3 (persistent blocks).  Host only. */
 mg_status mg_level_pass_kernel(const mg_handle* h, int level, int* kernel);

@@ -220,6 +220,17 @@ bool host_constrained(const HostLevel& L, int64_t g) {
   return false;
 }
 
+// Passes of one launch of a line sweep (linepass.cuh).
+constexpr int LINE_RUN = 5;
+
+// Whether smoothing on level j runs as line sweeps: not with the additive
+// variant, the boundary-vertex patches (which follow every colour) or a cap on
+// the grid (mg_set_block_limit caps the persistent colour passes).
+bool line_sweeps(const mg_handle* h, int j) {
+  const HostLevel& L = h->lv[j];
+  return L.line && h->additive == 0.0 && L.max_blocks == 0 && L.bnv == 0;
+}
+
 // `steps` smoothing steps on level j for nrhs vectors x, b (acc: a level
 // vector of scratch for the additive variant).  Multiplicative (the paper's,
 // Sec. 3.3): colours 0..C-1, C-2..0 per step.  A step ends and the next one
@@ -243,6 +254,27 @@ mg_status smooth_steps(mg_handle* h, int j, void* x, const void* b, void* acc, i
       launch_add_clear(h->f32(), x, acc, L.ndof * nrhs, stream);
       ++h->launches;
     }
+    return MG_OK;
+  }
+  if (line_sweeps(h, j)) {
+    // runs of passes whose colours differ in the x digit only: one launch each
+    int cross = -1, ns = 0, cx[LINE_RUN];
+    auto flush = [&]() {
+      if (ns > 0) {
+        h->ops->line_sweep(L, cross, ns, cx, L.sprec, x, b, h->d_fail, nrhs, stream);
+        ++h->launches;
+      }
+      ns = 0;
+    };
+    for (int s = 0; s < steps; ++s)
+      for (int t = (s > 0 ? 1 : 0); t < 2 * C - 1; ++t) {
+        const int col = t < C ? t : 2 * C - 2 - t;
+        if (L.count[col] == 0) continue;
+        if (col / 3 != cross || ns == LINE_RUN) flush();
+        cross = col / 3;
+        cx[ns++] = col % 3;
+      }
+    flush();
     return MG_OK;
   }
   for (int s = 0; s < steps; ++s) {
@@ -340,6 +372,19 @@ mg_status time_smoothing(mg_handle* h, int j, int nrhs, int steps, int reps, flo
 // blocks with every right-hand side on its own; 9, 10 the block kernel with
 // 2 or 8 threads per patch row.
 mg_status tune_passes(mg_handle* h, int mode, int nrhs) {
+  // the candidates are colour passes, one launch each
+  struct LinesOff {
+    std::vector<std::pair<int*, int>> was;
+    explicit LinesOff(mg_handle* hh) {
+      for (auto& L : hh->lv) {
+        was.push_back({&L.line, L.line});
+        L.line = 0;
+      }
+    }
+    ~LinesOff() {
+      for (auto& w : was) *w.first = w.second;
+    }
+  } lines_off(h);
   static std::mutex mu;
   static std::map<std::vector<int>, int> cache;
   const int64_t l0 = h->launches;
@@ -553,6 +598,7 @@ mg_status refine_in_cycle(mg_handle* h, int nrhs) {
   float best = 0.f;
   bool timed_once = false;
   for (int j = h->J; j > h->Ls && j >= 1; --j) {
+    if (line_sweeps(h, j)) continue;   // no colour passes of their own in the cycle
     const Pick& a = timed[j];
     const Pick& r = rule[j];
     const bool single = nrhs < 4;
@@ -814,6 +860,10 @@ static mg_status setup_internal(const mg_problem* p, void* cuda_stream, int nrhs
       }
     }
   }
+  // the kernel choices left to the library smooth by line sweeps
+  for (int j = 1; j <= J; ++j)
+    h->lv[j].line = (p->pass_kernel == 0 || p->pass_kernel == 4 || p->pass_kernel == 5) &&
+                    h->ops->line_fits(h->lv[j], h->lv[j].sprec);
   if ((st = tune_passes(h, p->pass_kernel, nrhs)) != MG_OK) return cleanup(st);
   h->main.nrhs = nrhs;
   h->nrhs = nrhs;
@@ -999,11 +1049,22 @@ mg_status mg_time_passes(mg_handle* h, int level, int kernel, double* us_per_pas
     return fail(MG_ERR_INVALID_ARG, "bad level, kernel or argument");
   HostLevel& L = h->lv[level];
   const int keep = L.pass_cta;
-  if (kernel > 0) L.pass_cta = std::max(kernel - 1, h->ops->warp_pass ? 0 : 1);
+  const int keep_line = L.line;
+  if (kernel > 0) {
+    L.pass_cta = std::max(kernel - 1, h->ops->warp_pass ? 0 : 1);
+    L.line = 0;
+  }
   float ms = 0.f;
   int64_t np = 0;
   const mg_status st = time_smoothing(h, level, h->nrhs, 2, 5, &ms, &np);
+  if (line_sweeps(h, level)) {   // colour passes of the two steps, several to a launch
+    np = 0;
+    const int C = num_colours(h->d);
+    for (int s = 0; s < 2; ++s)
+      for (int t = (s > 0 ? 1 : 0); t < 2 * C - 1; ++t) np += L.count[t < C ? t : 2 * C - 2 - t] > 0;
+  }
   L.pass_cta = keep;
+  L.line = keep_line;
   if (st != MG_OK) return st;
   *us_per_pass = np > 0 ? 1e3 * ms / (double)np : 0.0;
   return MG_OK;

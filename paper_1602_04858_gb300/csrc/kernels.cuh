@@ -1139,6 +1139,7 @@ __global__ void __launch_bounds__(NTH) k_bpatch_pass(const Lvl<D, K, T> L, const
 }  // namespace mgd
 
 #include "passcta.cuh"
+#include "linepass.cuh"
 
 namespace mgd {
 

@@ -489,12 +489,201 @@ void colour_pass(const HostLevel& h, int colour, int prec, const void* S, void* 
   else colour_pass_t<float, __nv_bfloat16>(h, colour, S, x, b, err, nrhs, s);
 }
 
+// Byte offset of the line-sweep tables: after the block-per-patch tables.
+template <typename T, typename TS>
+constexpr size_t line_tables_offset() {
+  return cta_tables_offset<T, TS, 8>() + al256(PassShapeC<D, K, T, TS, 1, 8>::TAB_BYTES);
+}
+
+// Registers per thread of the line-sweep kernel, and SMs of the device.
+template <typename T, typename TS, int NR>
+int line_regs() {
+  static std::atomic<int> regs[64];
+  return per_device_int(regs, [] {
+    cudaFuncAttributes a = {};
+    cudaFuncGetAttributes(&a, k_line_sweep<D, K, T, TS, NR>);
+    return a.numRegs > 0 ? a.numRegs : 128;
+  });
+}
+int num_sms() {
+  static std::atomic<int> sms[64];
+  return per_device_int(sms, [] {
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return nsm > 0 ? nsm : 152;
+  });
+}
+
+// Blocks per line (cluster size), teams per block and buffers per team of a line
+// sweep: the split with the smallest estimated time, in clocks, of a run of four
+// passes.  A pass takes a block its rounds of items: a fixed part (chain of
+// dependent work), then what the items of the blocks sharing an SM need of its
+// units or of the memory (about 25 bytes per clock and SM from HBM, 60 from L2;
+// FP64: at least one item's work on one of the SM's four partitions); ordering
+// the passes takes about 900 clocks between blocks, 150 within one.  Blocks that
+// start only when others leave add their start (8,000).  The clusters of one
+// block per SM that fit the device at once follow from eight groups of SMs.
+// Measured per pass (us): 2-D RT_1 256^2 3 x 6 7.25 (1 x 11 8.9, 6 x 7 8.2, 6 x 2
+// 8.2), 128^2 6 x 7 2.70 (3 x 8 2.99), 64^2 6 x 4 1.69 (7 x 3 and 1 x 11 above
+// 2.2); 3-D RT_0 64^3 1 x 11 4.6 (2 x 4 5.3); FP64 RT_1 256^2 3 x 7 50.1.
+struct LineSplit { int cl, teams, nsb, px, pc; size_t smem; };
+template <typename T, typename TS, int NR>
+LineSplit line_split(const HostLevel& h, int groups) {
+  using C = LineShape<D, K, T, TS, NR>;
+  const int nx = h.n - 1, sms = num_sms();
+  int64_t lines = groups;   // of the largest class
+  for (int e = 1; e < D; ++e) lines *= (nx + 2) / 3;
+  // the launches of one level follow one another: the last answer is kept
+  struct Memo { int n = 0, sms = 0, stream = 0; int64_t lines = 0; LineSplit q = {}; };
+  static thread_local Memo memo;
+  if (memo.n == h.n && memo.lines == lines && memo.sms == sms && memo.stream == h.s_evict_first) return memo.q;
+  const int regs = (line_regs<T, TS, NR>() + 7) / 8 * 8;
+  const double mem = (double)C::GPW * C::S_BYTES / (h.s_evict_first ? 25.0 : 60.0);
+  const double work = std::max((double)C::WORK, mem);
+  LineSplit best = {};
+  double best_t = 0.0;
+  for (int cl = 1; cl <= 8 && (cl == 1 || nx / cl >= 3); ++cl) {
+    const int m = (nx + cl - 1) / cl;
+    for (int teams = 1; teams * C::TT <= C::MAXT; ++teams) {
+      LineSplit q;
+      q.cl = cl;
+      q.teams = teams;
+      q.px = line_pitch<D, K>((m + 3) * (K + 1) + 1);
+      q.pc = m + 3;
+      int occ = 0;
+      for (int nsb = 2; nsb <= 3; ++nsb) {   // a third buffer where it costs no resident block
+        const size_t smem = C::layout(q.px, q.pc, teams, nsb).bytes;
+        const int threads = teams * C::TT + 32;
+        const int o = (int)std::min<int64_t>({(int64_t)(227 * 1024 / (smem + 1024)), 65536 / (regs * threads), 2048 / threads, 32});
+        if (nsb == 3 && o < occ) break;
+        occ = o;
+        q.nsb = nsb;
+        q.smem = smem;
+      }
+      if (occ < 1) continue;
+      const int64_t layer = cl == 1 ? sms : std::max(1, sms / 8 / cl * 8);   // clusters at one block per SM
+      const int64_t waves = (lines + layer * occ - 1) / (layer * occ);
+      const int64_t conc = std::min<int64_t>(occ, (lines + layer - 1) / layer);
+      const double items = (double)nx / cl / 3.0 / C::GPW;   // per pass and block
+      const double rounds = std::max(1.0, std::ceil(items / teams - 0.06));
+      const double busy = conc * std::min((double)teams, items) * work;
+      const double item = C::CHAIN + std::max(busy, sizeof(T) == 8 ? 4.0 * C::WORK : 0.0);
+      const double t = 8000.0 * waves + waves * 4.0 * (rounds * item + (cl > 1 ? 900.0 : 150.0));
+      if (best.cl == 0 || t < best_t) {
+        best = q;
+        best_t = t;
+      }
+    }
+  }
+  memo.n = h.n;
+  memo.lines = lines;
+  memo.sms = sms;
+  memo.stream = h.s_evict_first;
+  memo.q = best;
+  return best;   // cl = 0: no split fits the shared memory
+}
+
+template <typename T, typename TS, int NR>
+void line_sweep_nr(const HostLevel& h, int cross, int ns, const int* cx, void* x, const void* b, int* err, int groups,
+                  cudaStream_t s) {
+  using C = LineShape<D, K, T, TS, NR>;
+  static std::atomic<unsigned long long> attr{0};
+  once_per_device(attr, [] {
+    cudaFuncSetAttribute(k_line_sweep<D, K, T, TS, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  });
+  LineArgs a = {};
+  int digit = cross;
+  a.nlines = 1;
+  for (int e = 1; e < D; ++e) {
+    const int r = digit % 3;
+    digit /= 3;
+    a.first[e - 1] = colour_first(r);
+    a.cnt[e - 1] = colour_count(h.n, r);
+    a.nlines *= a.cnt[e - 1];
+  }
+  if (a.nlines == 0) return;
+  for (int c = 0; c < 3; ++c) {
+    a.cntx[c] = colour_count(h.n, c);
+    a.S[c] = h.S[c + 3 * cross];
+    a.s_prob[c] = h.s_prob[c + 3 * cross];
+  }
+  a.ns = ns;
+  for (int q = 0; q < ns; ++q) {
+    a.cx[q] = cx[q];
+    bool again = false;
+    for (int p = q + 1; p < ns; ++p) again = again || cx[p] == cx[q];
+    if (h.s_evict_first && !again) a.stream |= 1u << q;
+  }
+  // patch rows whose nodes lie in the patch's lower cell along x (nodes on the
+  // face between count to the upper cell)
+  for (int l = 0; l < C::NV; ++l) {
+    int vv[D], idx[D];
+    for (int e = 0; e < D; ++e) vv[e] = 2;
+    patch_local_decode<D, K>(vv, l, idx);
+    if (idx[0] < vv[0] * (K + 1)) ++a.nlo;
+    else ++a.nhi;
+  }
+  const LineSplit sp = line_split<T, TS, NR>(h, groups);
+  a.cl = sp.cl;
+  a.px = sp.px;
+  a.pc = sp.pc;
+  a.teams = sp.teams;
+  a.nsb = sp.nsb;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(a.nlines * sp.cl), groups);
+  cfg.blockDim = dim3(C::TT * sp.teams + 32);
+  cfg.dynamicSmemBytes = sp.smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)sp.cl;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = sp.cl > 1 ? 2 : 1;
+  const unsigned char* tabs = (const unsigned char*)h.R0 + line_tables_offset<T, TS>();
+  cudaLaunchKernelEx(&cfg, k_line_sweep<D, K, T, TS, NR>, mk<T>(h), a, tabs, (T*)x, (const T*)b, err, h.wait_ns,
+                     h.ndof, pstride(h, -1));
+}
+
+template <typename T, typename TS>
+void line_sweep_t(const HostLevel& h, int cross, int ns, const int* cx, void* x, const void* b, int* err, int nrhs,
+                  cudaStream_t s) {
+  const int g4 = (h.rhs_group < 4 || (h.rhs_prob > 0 && h.rhs_prob % 4 != 0)) ? 0 : nrhs / 4, rest = nrhs - 4 * g4;
+  const size_t off = (size_t)4 * g4 * h.ndof;
+  if (g4 > 0) line_sweep_nr<T, TS, 4>(h, cross, ns, cx, x, b, err, g4, s);
+  if (rest > 0) line_sweep_nr<T, TS, 1>(h, cross, ns, cx, (T*)x + off, (const T*)b + off, err, rest, s);
+}
+
+void line_sweep(const HostLevel& h, int cross, int ns, const int* cx, int prec, void* x, const void* b, int* err,
+                int nrhs, cudaStream_t s) {
+  if (prec == P64) line_sweep_t<double, double>(h, cross, ns, cx, x, b, err, nrhs, s);
+  else if (prec == P32) line_sweep_t<float, float>(h, cross, ns, cx, x, b, err, nrhs, s);
+  else line_sweep_t<float, __nv_bfloat16>(h, cross, ns, cx, x, b, err, nrhs, s);
+}
+
+template <typename T, typename TS>
+bool line_fits_t(const HostLevel& h) {
+  return line_split<T, TS, 4>(h, 1).cl > 0 && line_split<T, TS, 1>(h, 1).cl > 0;
+}
+
+int line_fits(const HostLevel& h, int prec) {
+  // RT_2 in FP64 keeps the colour passes: its product has no lanes to spare and
+  // one team per SM (26.5 against 22.7 us per pass on 64^2, 12.4 against 7.6 on 32^2)
+  if (prec == P64) return K < 2 && line_fits_t<double, double>(h);
+  if (prec == P32) return line_fits_t<float, float>(h);
+  return line_fits_t<float, __nv_bfloat16>(h);
+}
+
 // Bytes of the per-level colour-pass tables: those of the warp-per-patch
 // pass (segments, lane plans, row maps), then those of the block-per-patch
-// pass (gather descriptors, block plans).
+// pass (gather descriptors, block plans), then those of the line sweep.
 template <typename T, typename TS>
 size_t tables_bytes() {
-  return cta_tables_offset<T, TS, 8>() + (PassShapeC<D, K, T, TS, 1, 8>::TAB_BYTES + 15) / 16 * 16;
+  return line_tables_offset<T, TS>() + LineShape<D, K, T, TS>::TAB_BYTES;
 }
 int64_t template_elems(int sprec) {
   size_t b;
@@ -506,13 +695,14 @@ int64_t template_elems(int sprec) {
 
 template <typename T, typename TS>
 int build_template_t(const HostLevel& h, void* tabs, cudaStream_t s, std::string* why) {
-  std::vector<unsigned char> blob, blob_4, blob_2, blob_8;
+  std::vector<unsigned char> blob, blob_4, blob_2, blob_8, blob_l;
   std::string msg;
   bool ok = true;
   if constexpr (WARP_PASS) ok = build_pass_tables<D, K, T, TS>(mk<T>(h), tab<T>(), blob, msg);
   if (!ok || !build_cta_tables<D, K, T, TS, 4>(mk<T>(h), tab<T>(), blob_4, msg) ||
       !build_cta_tables<D, K, T, TS, 2>(mk<T>(h), tab<T>(), blob_2, msg) ||
-      !build_cta_tables<D, K, T, TS, 8>(mk<T>(h), tab<T>(), blob_8, msg)) {
+      !build_cta_tables<D, K, T, TS, 8>(mk<T>(h), tab<T>(), blob_8, msg) ||
+      !build_line_tables<D, K, T, TS>(mk<T>(h), tab<T>(), blob_l, msg)) {
     if (why) *why = "colour-pass tables of the " + std::to_string(h.n) + "^" + std::to_string(D) + " level: " + msg;
     return 1;
   }
@@ -520,6 +710,7 @@ int build_template_t(const HostLevel& h, void* tabs, cudaStream_t s, std::string
   std::memcpy(blob.data() + cta_tables_offset<T, TS, 4>(), blob_4.data(), blob_4.size());
   std::memcpy(blob.data() + cta_tables_offset<T, TS, 2>(), blob_2.data(), blob_2.size());
   std::memcpy(blob.data() + cta_tables_offset<T, TS, 8>(), blob_8.data(), blob_8.size());
+  std::memcpy(blob.data() + line_tables_offset<T, TS>(), blob_l.data(), blob_l.size());
   if (cudaMemcpyAsync(tabs, blob.data(), blob.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     if (why) *why = "upload of the colour-pass tables failed";
@@ -651,6 +842,7 @@ int plan_selftest_t(int n, double mu, std::string& why) {
   int r = check_cta_tables<D, K, T, TS, 4>(mk<T>(h), tab<T>(), why);
   if (r == 0) r = check_cta_tables<D, K, T, TS, 2>(mk<T>(h), tab<T>(), why);
   if (r == 0) r = check_cta_tables<D, K, T, TS, 8>(mk<T>(h), tab<T>(), why);
+  if (r == 0) r = check_line_tables<D, K, T, TS>(mk<T>(h), tab<T>(), why);
   if (r != 0) return r;
   return check_row_plans(h, why);
 }
@@ -840,6 +1032,8 @@ DKOps make_ops() {
   o.patch_setup = patch_setup;
   o.colour_pass = colour_pass;
   o.additive_pass = additive_pass;
+  o.line_sweep = line_sweep;
+  o.line_fits = line_fits;
   o.coarse_assemble = coarse_assemble;
   o.copy_constrained = copy_constrained;
   o.residual_norm = residual_norm;

@@ -81,6 +81,8 @@ struct HostLevel {
                          // are resident)
   int cta_tpr;           // threads per patch row of the block-per-patch pass for single right-hand
                          // sides: 4, 2 or 8
+  int line;              // 1: smoothing runs as line sweeps (linepass.cuh), the passes of one class of
+                         // vertex lines per launch, instead of one launch per colour pass
   int rhs_group;         // right-hand sides sharing each S_v load in the colour passes: 4 (groups
                          // of four where the count allows) or 1 (every right-hand side on its own)
   // problems of one shape stored one after another (grouped batches): rhs_prob
@@ -121,6 +123,12 @@ struct DKOps {
                     cudaStream_t);
   void (*prolong_add)(const HostLevel& Lf, const HostLevel& Lc, int f32, const void* xc, void* xf, int nrhs,
                       cudaStream_t);
+  // ns consecutive colour passes of the class of vertex lines `cross` (colour =
+  // x digit + 3 cross), x digits cx[0 .. ns), in one launch
+  void (*line_sweep)(const HostLevel&, int cross, int ns, const int* cx, int prec, void* x, const void* b, int* err,
+                     int nrhs, cudaStream_t);
+  // whether the level's strips fit the line sweep's shared memory
+  int (*line_fits)(const HostLevel&, int prec);
   // patch inverses of one colour into S (storage precision sprec); *fail set on a zero pivot
   void (*patch_setup)(const HostLevel&, int colour, int sprec, void* S, int* fail, cudaStream_t);
   // one colour pass in precision prec on vectors x, b; a timed-out wait for
