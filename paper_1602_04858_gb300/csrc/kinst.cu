@@ -496,12 +496,12 @@ constexpr size_t line_tables_offset() {
 }
 
 // Registers per thread of the line-sweep kernel, and SMs of the device.
-template <typename T, typename TS, int NR>
+template <typename T, typename TS, int NR, int MB>
 int line_regs() {
   static std::atomic<int> regs[64];
   return per_device_int(regs, [] {
     cudaFuncAttributes a = {};
-    cudaFuncGetAttributes(&a, k_line_sweep<D, K, T, TS, NR>);
+    cudaFuncGetAttributes(&a, k_line_sweep<D, K, T, TS, NR, MB>);
     return a.numRegs > 0 ? a.numRegs : 128;
   });
 }
@@ -515,46 +515,56 @@ int num_sms() {
   });
 }
 
+// Shared-memory limit of the line-sweep kernel, set once per device.
+template <typename T, typename TS, int NR, int MB>
+void line_attr() {
+  static std::atomic<unsigned long long> attr{0};
+  once_per_device(attr, [] {
+    cudaFuncSetAttribute(k_line_sweep<D, K, T, TS, NR, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  });
+}
+
 // Blocks per line (cluster size), teams per block and buffers per team of a line
-// sweep: the split with the smallest estimated time, in clocks, of a run of four
-// passes.  A pass takes a block its rounds of items: a fixed part (chain of
-// dependent work), then what the items of the blocks sharing an SM need of its
-// units or of the memory (about 25 bytes per clock and SM from HBM, 60 from L2;
-// FP64: at least one item's work on one of the SM's four partitions); ordering
-// the passes takes about 900 clocks between blocks, 150 within one.  Blocks that
-// start only when others leave add their start (8,000).  The clusters of one
-// block per SM that fit the device at once follow from eight groups of SMs.
-// Measured per pass (us): 2-D RT_1 256^2 3 x 6 7.25 (1 x 11 8.9, 6 x 7 8.2, 6 x 2
-// 8.2), 128^2 6 x 7 2.70 (3 x 8 2.99), 64^2 6 x 4 1.69 (7 x 3 and 1 x 11 above
-// 2.2); 3-D RT_0 64^3 1 x 11 4.6 (2 x 4 5.3); FP64 RT_1 256^2 3 x 7 50.1.
-struct LineSplit { int cl, teams, nsb, px, pc; size_t smem; };
-template <typename T, typename TS, int NR>
-LineSplit line_split(const HostLevel& h, int groups) {
+// sweep: the split with the smallest estimated time of a run of four passes.  A
+// pass takes a block its rounds of items: a fixed part (chain of dependent work,
+// 1,000 units), then what the items of the blocks sharing an SM need of its units
+// (half a WORK each; FP64 at least 2.5 times one item's work, its partition's share)
+// or of the memory (a unit per 42 bytes and SM); ordering the passes costs 1,300
+// between blocks.  Every wave of blocks costs a start (29,000, and 20 per strip entry
+// of a thread), which hides less behind the launch before where the two do not fit
+// the device together (2,000).  How many clusters the device holds at once is asked
+// of the occupancy interface, since clusters do not cross the groups of SMs (of 3:
+// 46 with one block per SM, of 4: 36, of 6: 23, of 8: 15); a split that needs a
+// second wave for a few lines loses a third or more.  The constants were fitted to
+// 4,000 measured splits of 43 levels (2-D RT_0 to RT_2, 3-D RT_0, FP32, FP64, BF16
+// inverses, 1 to 16 right-hand sides): the rule's splits take 2 % longer than the
+// best ones on average, 12 % at most.  Measured per pass (us): RT_1 256^2 3 x 6 7.2
+// (3 x 5 7.6, 6 x 7 8.2), FP64 3 x 6 49.3 (6 x 7 56.3); 128^2 6 x 7 2.74 (3 x 8
+// 2.99); 64^2 1.68 (1 x 11 above 2.2); 192^2 BF16 inverses 2 x 11 4.8 (6 x 4 4.3);
+// RT_0 128^2 1 x 11 1.31 (2 x 6 1.68); 3-D RT_0 64^3 1 x 11 4.5 (1 x 10 4.8), 32^3
+// 1 x 12 1.45 (1 x 11 of the other form 1.73).  The form of the kernel (LEAN) is
+// chosen the same way, by how many lines fit at once.
+struct LineSplit { int cl, teams, nsb, mb, px, pc; size_t smem; double t; };
+template <typename T, typename TS, int NR, int MB>
+void line_split_form(int nx, int sms, int64_t lines, LineSplit& best) {
   using C = LineShape<D, K, T, TS, NR>;
-  const int nx = h.n - 1, sms = num_sms();
-  int64_t lines = groups;   // of the largest class
-  for (int e = 1; e < D; ++e) lines *= (nx + 2) / 3;
-  // the launches of one level follow one another: the last answer is kept
-  struct Memo { int n = 0, sms = 0, stream = 0; int64_t lines = 0; LineSplit q = {}; };
-  static thread_local Memo memo;
-  if (memo.n == h.n && memo.lines == lines && memo.sms == sms && memo.stream == h.s_evict_first) return memo.q;
-  const int regs = (line_regs<T, TS, NR>() + 7) / 8 * 8;
-  const double mem = (double)C::GPW * C::S_BYTES / (h.s_evict_first ? 25.0 : 60.0);
-  const double work = std::max((double)C::WORK, mem);
-  LineSplit best = {};
-  double best_t = 0.0;
+  line_attr<T, TS, NR, MB>();
+  const int regs = (line_regs<T, TS, NR, MB>() + 7) / 8 * 8;
+  const double work = std::max(0.5 * C::WORK, (double)C::GPW * C::S_BYTES / 42.0);
+  const double chain = K == 2 ? 2000.0 : 1000.0, start = 29000.0;
   for (int cl = 1; cl <= 8 && (cl == 1 || nx / cl >= 3); ++cl) {
     const int m = (nx + cl - 1) / cl;
     for (int teams = 1; teams * C::TT <= C::MAXT; ++teams) {
       LineSplit q;
       q.cl = cl;
       q.teams = teams;
+      q.mb = MB;
       q.px = line_pitch<D, K>((m + 3) * (K + 1) + 1);
       q.pc = m + 3;
-      int occ = 0;
+      int occ = 0;   // blocks on an SM
+      const int threads = teams * C::TT + 32;
       for (int nsb = 2; nsb <= 3; ++nsb) {   // a third buffer where it costs no resident block
         const size_t smem = C::layout(q.px, q.pc, teams, nsb).bytes;
-        const int threads = teams * C::TT + 32;
         const int o = (int)std::min<int64_t>({(int64_t)(227 * 1024 / (smem + 1024)), 65536 / (regs * threads), 2048 / threads, 32});
         if (nsb == 3 && o < occ) break;
         occ = o;
@@ -562,36 +572,64 @@ LineSplit line_split(const HostLevel& h, int groups) {
         q.smem = smem;
       }
       if (occ < 1) continue;
-      const int64_t layer = cl == 1 ? sms : std::max(1, sms / 8 / cl * 8);   // clusters at one block per SM
-      const int64_t waves = (lines + layer * occ - 1) / (layer * occ);
-      const int64_t conc = std::min<int64_t>(occ, (lines + layer - 1) / layer);
       const double items = (double)nx / cl / 3.0 / C::GPW;   // per pass and block
-      const double rounds = std::max(1.0, std::ceil(items / teams - 0.06));
+      const double rounds = std::max(1.0, std::ceil(items / teams - 0.03));
+      const int64_t conc = std::min<int64_t>(occ, (lines * cl + sms - 1) / sms);
       const double busy = conc * std::min((double)teams, items) * work;
-      const double item = C::CHAIN + std::max(busy, sizeof(T) == 8 ? 4.0 * C::WORK : 0.0);
-      const double t = 8000.0 * waves + waves * 4.0 * (rounds * item + (cl > 1 ? 900.0 : 150.0));
-      if (best.cl == 0 || t < best_t) {
-        best = q;
-        best_t = t;
+      const double item = chain + std::max(busy, sizeof(T) == 8 ? 2.5 * C::WORK : 0.0);
+      const int strip = (C::R::XROWS + C::R::BROWS) * ((m + 3) * (K + 1) + 1) * NR;
+      const double run = start + 20.0 * ((strip + teams * C::TT - 1) / (teams * C::TT)) +
+                         4.0 * (rounds * item + (cl > 1 ? 1300.0 : 0.0));
+      if (best.cl > 0 && run > best.t) continue;
+      int slots = occ * sms;   // lines the device holds at once
+      if (cl > 1) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(cl);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = q.smem;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)cl;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&slots, k_line_sweep<D, K, T, TS, NR, MB>, &cfg) != cudaSuccess) {
+          cudaGetLastError();
+          continue;
+        }
+        if (slots < 1) continue;
       }
+      // a last wave that is not full ends sooner
+      const double w = (double)lines / slots;
+      q.t = (run + (2 * lines > slots ? 2000.0 : 0.0)) * (w <= 1.0 ? 1.0 : 0.7 * std::ceil(w) + 0.3 * w);
+      if (best.cl == 0 || q.t < best.t || (q.t == best.t && q.cl == best.cl && MB == best.mb)) best = q;
     }
   }
-  memo.n = h.n;
-  memo.lines = lines;
-  memo.sms = sms;
-  memo.stream = h.s_evict_first;
-  memo.q = best;
+}
+template <typename T, typename TS, int NR>
+LineSplit line_split(const HostLevel& h, int groups) {
+  const int nx = h.n - 1, sms = num_sms();
+  int64_t lines = groups;   // of the largest class
+  for (int e = 1; e < D; ++e) lines *= (nx + 2) / 3;
+  // the launches of a hierarchy repeat: each thread keeps its last few answers
+  struct Memo { int n = 0, sms = 0; int64_t lines = 0; LineSplit q = {}; };
+  static thread_local Memo memo[16];
+  static thread_local int next = 0;
+  for (const Memo& m : memo)
+    if (m.n == h.n && m.lines == lines && m.sms == sms) return m.q;
+  LineSplit best = {};
+  line_split_form<T, TS, NR, 1>(nx, sms, lines, best);
+  if constexpr (LineShape<D, K, T, TS, NR>::LEAN) line_split_form<T, TS, NR, 2>(nx, sms, lines, best);
+  memo[next] = {h.n, sms, lines, best};
+  next = (next + 1) % 16;
   return best;   // cl = 0: no split fits the shared memory
 }
 
 template <typename T, typename TS, int NR>
-void line_sweep_nr(const HostLevel& h, int cross, int ns, const int* cx, void* x, const void* b, int* err, int groups,
-                  cudaStream_t s) {
+void line_sweep_nr(const HostLevel& h, int cross, int ns, const int* cx, void* x, const void* b, int* err,
+                   int groups, cudaStream_t s) {
   using C = LineShape<D, K, T, TS, NR>;
-  static std::atomic<unsigned long long> attr{0};
-  once_per_device(attr, [] {
-    cudaFuncSetAttribute(k_line_sweep<D, K, T, TS, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  });
   LineArgs a = {};
   int digit = cross;
   a.nlines = 1;
@@ -645,8 +683,12 @@ void line_sweep_nr(const HostLevel& h, int cross, int ns, const int* cx, void* x
   cfg.attrs = at;
   cfg.numAttrs = sp.cl > 1 ? 2 : 1;
   const unsigned char* tabs = (const unsigned char*)h.R0 + line_tables_offset<T, TS>();
-  cudaLaunchKernelEx(&cfg, k_line_sweep<D, K, T, TS, NR>, mk<T>(h), a, tabs, (T*)x, (const T*)b, err, h.wait_ns,
-                     h.ndof, pstride(h, -1));
+  auto launch = [&](auto kernel) {
+    cudaLaunchKernelEx(&cfg, kernel, mk<T>(h), a, tabs, (T*)x, (const T*)b, err, h.wait_ns, h.ndof, pstride(h, -1));
+  };
+  if constexpr (C::LEAN)
+    if (sp.mb == 2) return launch(k_line_sweep<D, K, T, TS, NR, 2>);
+  launch(k_line_sweep<D, K, T, TS, NR, 1>);
 }
 
 template <typename T, typename TS>

@@ -240,11 +240,15 @@ struct LineShape {
   // largest block (without the copying warp): what the inverse buffers leave
   // room for, and registers for the plan
   static constexpr int MAXT = K == 2 ? (sizeof(T) == 4 ? 288 : 192) : (K == 1 ? (sizeof(T) == 4 && NR == 1 ? 384 : 256) : 512);
+  // 3-D RT_0 in FP32 with one right-hand side comes in two forms: with the registers
+  // of one of the largest blocks on an SM (96: all its loads in flight at once;
+  // 16^3 1.02 us a pass, 32^3 1.59) and with those of two (56, more lines at once;
+  // 1.15, 1.44).  2-D RT_0 is faster with 96 throughout (512^2 4.0 against 4.8)
+  static constexpr bool LEAN = D == 3 && K == 0 && sizeof(T) == 4 && NR == 1;
   // clocks of an SM that one item (GPW patches) takes of its busiest unit besides
   // the copies: shared-memory wavefronts, or the FP64 units (two FMAs per clock)
   static constexpr int WORK = sizeof(T) == 8 ? 16 * TW * NR * (NS + JCH * PR + 10)
                                              : TW * (NS * (NR == 1 ? 7 : 16) / 4 + JCH * (RG * (int)sizeof(TS) / 4 + 1) + 20 * NR);
-  static constexpr int CHAIN = K == 2 ? 1200 : 600;   // clocks of an item's dependent work outside those units
   // scratch per patch (T): residual ((r, r) pairs with one FP32 right-hand side), FP64 partial sums
   static constexpr int RP = (sizeof(T) == 4 && NR == 1) ? 2 : NR;
   static constexpr int O_D = (NV * RP + 3) / 4 * 4;
@@ -754,8 +758,9 @@ __device__ __forceinline__ void load_rows(const TS* p, T (&o)[PR]) {
   }
 }
 
-template <int D, int K, typename T, typename TS, int NR>
-__global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32)
+// MB: blocks per SM that the registers leave room for (2: LineShape::LEAN)
+template <int D, int K, typename T, typename TS, int NR, int MB>
+__global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
     k_line_sweep(const __grid_constant__ Lvl<D, K, T> L, const __grid_constant__ LineArgs A,
                  const unsigned char* __restrict__ tabs, T* x, const T* __restrict__ b, int* __restrict__ err,
                  uint64_t wait_ns, int64_t vs, const ProbStride ps) {
@@ -766,6 +771,7 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32)
   constexpr int EB = NR * (int)sizeof(T);   // bytes of a strip entry (the right-hand sides together)
   constexpr uint64_t NB_LIMIT = 4000000000ull;   // bound of the waits for the neighbour blocks (ns)
   extern __shared__ __align__(128) unsigned char smem[];
+  pdl_launch_dependents();   // the next launch's blocks prepare beside this one's
   const int tid = threadIdx.x;
   const int N = A.teams * C::TT;            // threads of the teams; the last warp copies the inverses
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, nw = N >> 5;
@@ -869,7 +875,6 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32)
       cluster_arrive();   // barriers ready
       cluster_wait();
     }
-    pdl_launch_dependents();
     // a buffer is refilled once its team has released it; the rest is given up
     // when a team has given up (or nothing moves for longer than any wait)
     uint64_t t0 = globaltimer_ns();
@@ -1017,7 +1022,6 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32)
     sofs[q] = e < ne ? (r * A.px + j) * EB : -1;
     gofs[q] = e < ne && base >= 0 && (unsigned)(x0 + j) < (unsigned)hi ? base + x0 + j : -1;
   }
-  pdl_launch_dependents();
   pdl_wait();   // x comes from the preceding kernel
 #pragma unroll
   for (int q = 0; q < PRE; ++q)
