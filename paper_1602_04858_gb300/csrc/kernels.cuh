@@ -9,6 +9,7 @@
 #include "device.cuh"
 #include "ops.h"
 #include "passplan.cuh"
+#include "factrow.cuh"
 #include "rowplan.cuh"
 
 namespace mgd {

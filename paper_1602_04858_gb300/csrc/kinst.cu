@@ -222,10 +222,23 @@ template <> RowPlans<float> plans<float>(const HostLevel& h) {
   return RowPlans<float>{h.rp.cls, h.rp.ptr, h.rp.mptr, h.rp.pe, h.rp.pcf32, h.rp.me, h.rp.mcf32};
 }
 
+// In 2-D and FP64 the operator's products are the bound (factrow.cuh); FP32 and 3-D
+// RT_0 (one node across a cell: little to factor out) keep the row plans.
+void fact_apply(const HostLevel& h, const double* x, const double* b, double* y, int zero_c, int nrhs, ProbStride ps,
+                cudaStream_t s) {
+  if constexpr (D == 2) {
+    const FactRowGrid fg = fact_row_grid<K>(h.n);
+    k_fact_apply<D, K><<<dim3((unsigned)fg.first[3], nrhs), 32 * FR_WARPS, 0, s>>>(mk<double>(h), tab<double>(), fg, x, b, y,
+                                                                              zero_c, h.ndof, ps);
+  }
+}
+
 void apply(const HostLevel& h, int f32, const void* x, void* y, int nrhs, cudaStream_t s) {
   const dim3 grid(blocks(h.ndof, 256), nrhs);
   if (f32)
     k_apply<D, K, float><<<grid, 256, 0, s>>>(mk<float>(h), plans<float>(h), (const float*)x, (float*)y, h.ndof);
+  else if constexpr (D == 2)
+    fact_apply(h, (const double*)x, nullptr, (double*)y, 0, nrhs, ProbStride{}, s);
   else
     k_apply<D, K, double><<<grid, 256, 0, s>>>(mk<double>(h), plans<double>(h), (const double*)x, (double*)y,
                                                h.ndof);
@@ -237,6 +250,8 @@ void residual(const HostLevel& h, int f32, const void* x, const void* b, void* r
   if (f32)
     k_residual<D, K, float><<<grid, 256, 0, s>>>(mk<float>(h), plans<float>(h), (const float*)x, (const float*)b,
                                                  (float*)r, zero_c, h.ndof, pstride(h, -1));
+  else if constexpr (D == 2)
+    fact_apply(h, (const double*)x, (const double*)b, (double*)r, zero_c, nrhs, pstride(h, -1), s);
   else
     k_residual<D, K, double><<<grid, 256, 0, s>>>(mk<double>(h), plans<double>(h), (const double*)x,
                                                   (const double*)b, (double*)r, zero_c, h.ndof, pstride(h, -1));
@@ -1031,11 +1046,20 @@ void coarse_assemble(const HostLevel& h, const int64_t* free_list, const int* g2
   k_coarse_assemble<D, K><<<1, 512, 0, s>>>(mk<double>(h), tab<double>(), free_list, g2l, nf, M, E);
 }
 
+int64_t residual_norm_count(const HostLevel& h) {
+  if constexpr (D == 2) return fact_row_grid<K>(h.n).first[3];
+  else return residual_norm_blocks(h.ndof);
+}
+
 int64_t residual_norm(const HostLevel& h, const double* x, const double* b, double* r, double* partial,
                       cudaStream_t s) {
-  const int64_t nb = residual_norm_blocks(h.ndof);
-  k_residual_norm_rp<D, K, double><<<(unsigned)nb, RN_THREADS, 0, s>>>(mk<double>(h), plans<double>(h), x, b, r,
-                                                                       partial);
+  const int64_t nb = residual_norm_count(h);
+  if constexpr (D == 2)
+    k_fact_residual_norm<D, K><<<(unsigned)nb, 32 * FR_WARPS, 0, s>>>(mk<double>(h), tab<double>(), fact_row_grid<K>(h.n), x, b,
+                                                                  r, partial);
+  else
+    k_residual_norm_rp<D, K, double><<<(unsigned)nb, RN_THREADS, 0, s>>>(mk<double>(h), plans<double>(h), x, b, r,
+                                                                         partial);
   return nb;
 }
 
@@ -1079,6 +1103,7 @@ DKOps make_ops() {
   o.coarse_assemble = coarse_assemble;
   o.copy_constrained = copy_constrained;
   o.residual_norm = residual_norm;
+  o.residual_norm_count = residual_norm_count;
   o.load_vector = load_vector;
   o.template_elems = template_elems;
   o.build_template = build_template;

@@ -161,6 +161,7 @@ struct DKOps {
                           double* E, cudaStream_t);
   // FP64 r = b - A x (r may be null) and per-block partial sums of |r|^2;
   // returns the number of partials (blocks) written
+  int64_t (*residual_norm_count)(const HostLevel&);   // partial sums that residual_norm writes
   int64_t (*residual_norm)(const HostLevel&, const double* x, const double* b, double* r, double* partial,
                            cudaStream_t);
   // load vector of cellwise-constant f (D x ncell) and g (ncell, may be null), FP64
@@ -199,7 +200,7 @@ void launch_scale_by_rnorm(const double* a, const double* n2, double* b, int64_t
 void launch_add_const(double* a, double s, int64_t n, cudaStream_t);
 // out[0] = sqrt(sum of partial[0..n)), fixed summation order, one block
 void launch_sqrt_sum(const double* partial, int64_t n, double* out, cudaStream_t);
-// number of partial sums k_residual_norm writes for a level of ndof dofs
+// number of partial sums k_residual_norm(_rp) writes for a level of ndof dofs
 inline int64_t residual_norm_blocks(int64_t ndof) { return (ndof + 255) / 256; }
 int multidot_blocks();
 // vectors r = 0..nc-1 of B (each ndof long) become the unit vectors e_{c0+r}
