@@ -628,13 +628,7 @@ mg_status vcycle_dev(mg_handle* h, const double* r, double* z) {
     ++h->launches;
   }
   TRY(vcycle_graph(h));
-  if (h->prec == P64) {
-    CU(cudaMemcpyAsync(z, L.X, n * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
-  } else {
-    launch_f2d((const float*)L.X, z, n, h->stream);
-    ++h->launches;
-  }
-  h->ops->copy_constrained(L, r, z, h->nrhs, h->stream);
+  h->ops->result(L, h->f32(), L.X, r, z, h->nrhs, h->stream);
   ++h->launches;
   CU(cudaGetLastError());
   return MG_OK;
@@ -1606,12 +1600,7 @@ mg_status sub_vcycle(mg_handle* h, const double* r, double* z, cudaStream_t s) {
     ++h->launches;
   }
   TRY(vcycle_level(h, h->J, h->main, true, s));
-  if (h->prec == P64) CU(cudaMemcpyAsync(z, L.X, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  else {
-    launch_f2d((const float*)L.X, z, n, s);
-    ++h->launches;
-  }
-  h->ops->copy_constrained(L, r, z, h->nrhs, s);
+  h->ops->result(L, h->f32(), L.X, r, z, h->nrhs, s);
   ++h->launches;
   return MG_OK;
 }
@@ -1810,14 +1799,8 @@ mg_status group_vcycle(mg_batch* B, int g, const double* r, double* z, cudaStrea
   }
   TRY(vcycle_level(gh, gh->J, gh->main, true, s));
   for (int i = 0; i < nseg; ++i) {
-    double* zi = z + B->off[mem[i]];
-    if (gh->prec == P64)
-      CU(cudaMemcpyAsync(zi, (double*)L.X + i * per, seg_len * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    else {
-      launch_f2d((const float*)L.X + i * per, zi, seg_len, s);
-      ++gh->launches;
-    }
-    gh->ops->copy_constrained(L, r + B->off[mem[i]], zi, (int)(seg_len / L.ndof), s);
+    gh->ops->result(L, gh->f32(), (const char*)L.X + i * per * gh->vbytes(), r + B->off[mem[i]], z + B->off[mem[i]],
+                    (int)(seg_len / L.ndof), s);
     ++gh->launches;
   }
   return MG_OK;

@@ -741,22 +741,10 @@ mg_status cnn_cuda(cudaError_t e, const char* what) {
                         std::string(what) + ": " + cudaGetErrorString(e));
 }
 
-// Launches of a pass follow one another: each may start while the one before ends
-// (it waits before it touches any data; the kernels read with plain loads through plain
-// pointers, which stay behind that wait).
+// Launches of a pass follow one another (launch_pdl).
 template <typename... KArgs, typename... Args>
 void chain(const mg_cnn* N, dim3 grid, int threads, size_t smem, void (*kernel)(KArgs...), Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = N->stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+  launch_pdl(kernel, grid, threads, smem, N->stream, args...);
 }
 
 // 3-plane convolution to 32 channels on the CUDA cores (k_conv3).

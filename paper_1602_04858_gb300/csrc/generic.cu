@@ -2,6 +2,7 @@
 // precision casts, the coarsest-level dense solve and the FP64 vector
 // kernels of the Krylov solver.
 #include "kernels.cuh"
+#include "async.cuh"
 #include "ops.h"
 
 namespace mgd {
@@ -51,7 +52,9 @@ __global__ void k_gauss_jordan(double* M, double* E, int n, int nrhs, int* fail)
 // Coarsest-level solve: x = 0, then x[free_i] = sum_j inv_ij b[free_j] (FP64 arithmetic).
 template <typename T>
 __global__ void k_coarse_apply(const double* __restrict__ inv, const int64_t* __restrict__ free_list, int nf,
-                               int64_t ndof, const T* __restrict__ b, T* __restrict__ x, int64_t vs) {
+                               int64_t ndof, const T* b, T* x, int64_t vs) {
+  pdl_wait();
+  pdl_launch_dependents();
   extern __shared__ double bs[];
   b += blockIdx.x * vs;   // one block per right-hand side
   x += blockIdx.x * vs;
@@ -193,8 +196,10 @@ constexpr int DENSE_THREADS = 256;
 // NR right-hand sides (vectors n apart) share each read of Bd.
 template <typename T, int NR>
 __global__ void __launch_bounds__(DENSE_THREADS) k_dense_partial(const T* __restrict__ Bd, int64_t n,
-                                                                 const T* __restrict__ b, T* __restrict__ partial,
-                                                                 int64_t bd_stride, int64_t bvs, int64_t pstride) {
+                                                                 const T* b, T* partial, int64_t bd_stride, int64_t bvs,
+                                                                 int64_t pstride) {
+  pdl_wait();
+  pdl_launch_dependents();
   Bd += blockIdx.z * bd_stride;
   b += blockIdx.z * bvs;
   partial += blockIdx.z * pstride;
@@ -228,13 +233,15 @@ __global__ void __launch_bounds__(DENSE_THREADS) k_dense_partial(const T* __rest
 }
 
 template <typename T>
-__global__ void k_dense_reduce(const T* __restrict__ partial, int chunks, int64_t n, T* __restrict__ z,
-                               int64_t zvs, int64_t pstride) {
+__global__ void k_dense_reduce(const T* partial, int chunks, int64_t n, T* z, int64_t zvs, int64_t pstride) {
+  pdl_wait();
+  pdl_launch_dependents();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   partial += blockIdx.z * pstride + (int64_t)blockIdx.y * chunks * n;   // one right-hand side per blockIdx.y
   z += blockIdx.z * zvs;
   T acc = T(0);
+#pragma unroll 16
   for (int y = 0; y < chunks; ++y) acc += partial[y * n + i];
   z[(int64_t)blockIdx.y * n + i] = acc;
 }
@@ -338,12 +345,16 @@ void dense_apply_t(const T* Bd, int64_t bd_stride, int64_t n, const T* b, T* z, 
     const int nr = (rhs - r0 < 4) ? rhs - r0 : 4;
     const dim3 grid(blocks(n, DENSE_THREADS), DENSE_CHUNKS, nprob);
     const T* bb = b + (int64_t)r0 * n;
-    if (nr == 4) k_dense_partial<T, 4><<<grid, DENSE_THREADS, 0, s>>>(Bd, n, bb, partial, bd_stride, vs, pstride);
-    else if (nr == 3) k_dense_partial<T, 3><<<grid, DENSE_THREADS, 0, s>>>(Bd, n, bb, partial, bd_stride, vs, pstride);
-    else if (nr == 2) k_dense_partial<T, 2><<<grid, DENSE_THREADS, 0, s>>>(Bd, n, bb, partial, bd_stride, vs, pstride);
-    else k_dense_partial<T, 1><<<grid, DENSE_THREADS, 0, s>>>(Bd, n, bb, partial, bd_stride, vs, pstride);
-    k_dense_reduce<T><<<dim3(blocks(n, 256), nr, nprob), 256, 0, s>>>(partial, DENSE_CHUNKS, n,
-                                                                      z + (int64_t)r0 * n, vs, pstride);
+    // (several problems: 1 % slower when the next launch comes up early)
+    auto run = [&](auto kernel, const dim3& g, auto... args) {
+      if (nprob == 1) launch_pdl(kernel, g, DENSE_THREADS, 0, s, args...);
+      else kernel<<<g, DENSE_THREADS, 0, s>>>(args...);
+    };
+    if (nr == 4) run(k_dense_partial<T, 4>, grid, Bd, n, bb, partial, bd_stride, vs, pstride);
+    else if (nr == 3) run(k_dense_partial<T, 3>, grid, Bd, n, bb, partial, bd_stride, vs, pstride);
+    else if (nr == 2) run(k_dense_partial<T, 2>, grid, Bd, n, bb, partial, bd_stride, vs, pstride);
+    else run(k_dense_partial<T, 1>, grid, Bd, n, bb, partial, bd_stride, vs, pstride);
+    run(k_dense_reduce<T>, dim3(blocks(n, DENSE_THREADS), nr, nprob), partial, DENSE_CHUNKS, n, z + (int64_t)r0 * n, vs, pstride);
   }
 }
 
@@ -392,8 +403,8 @@ void launch_gauss_jordan(double* M, double* E, int n, int nrhs, int* fail, cudaS
 void launch_coarse_apply(const double* inv, const int64_t* free_list, int nf, int64_t ndof, int f32, const void* b,
                          void* x, int nrhs, cudaStream_t s) {
   const size_t smem = sizeof(double) * (size_t)nf;
-  if (f32) k_coarse_apply<float><<<nrhs, 512, smem, s>>>(inv, free_list, nf, ndof, (const float*)b, (float*)x, ndof);
-  else k_coarse_apply<double><<<nrhs, 512, smem, s>>>(inv, free_list, nf, ndof, (const double*)b, (double*)x, ndof);
+  if (f32) launch_pdl(k_coarse_apply<float>, nrhs, 512, smem, s, inv, free_list, nf, ndof, (const float*)b, (float*)x, ndof);
+  else launch_pdl(k_coarse_apply<double>, nrhs, 512, smem, s, inv, free_list, nf, ndof, (const double*)b, (double*)x, ndof);
 }
 
 int multidot_blocks() { return MD_BLOCKS; }

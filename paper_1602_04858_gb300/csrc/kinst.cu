@@ -222,39 +222,61 @@ template <> RowPlans<float> plans<float>(const HostLevel& h) {
   return RowPlans<float>{h.rp.cls, h.rp.ptr, h.rp.mptr, h.rp.pe, h.rp.pcf32, h.rp.me, h.rp.mcf32};
 }
 
-// In 2-D and FP64 the operator's products are the bound (factrow.cuh); FP32 and 3-D
-// RT_0 (one node across a cell: little to factor out) keep the row plans.
-void fact_apply(const HostLevel& h, const double* x, const double* b, double* y, int zero_c, int nrhs, ProbStride ps,
-                cudaStream_t s) {
-  if constexpr (D == 2) {
+// The operator in FP64.  In 2-D its products are the bound (factrow.cuh: 59 us for the
+// residual norm of 320^2 RT_1, row plans 87); FP32 and 3-D RT_0 (one node across a
+// cell: little to factor out) keep the row plans.
+template <int DD>
+void apply64(const HostLevel& h, const double* x, double* y, int nrhs, cudaStream_t s) {
+  if constexpr (DD == 2) {
     const FactRowGrid fg = fact_row_grid<K>(h.n);
-    k_fact_apply<D, K><<<dim3((unsigned)fg.first[3], nrhs), 32 * FR_WARPS, 0, s>>>(mk<double>(h), tab<double>(), fg, x, b, y,
-                                                                              zero_c, h.ndof, ps);
+    k_fact_apply<DD, K><<<dim3((unsigned)fg.first[3], nrhs), 32 * FR_WARPS, 0, s>>>(mk<double>(h), tab<double>(), fg,
+        x, (const double*)nullptr, y, 0, h.ndof, ProbStride{});
+  } else {
+    k_apply<DD, K, double><<<dim3(blocks(h.ndof, 256), nrhs), 256, 0, s>>>(mk<double>(h), plans<double>(h), x, y,
+        h.ndof);
+  }
+}
+template <int DD>
+void residual64(const HostLevel& h, const double* x, const double* b, double* r, int zero_c, int nrhs, cudaStream_t s) {
+  if constexpr (DD == 2) {
+    const FactRowGrid fg = fact_row_grid<K>(h.n);
+    k_fact_apply<DD, K><<<dim3((unsigned)fg.first[3], nrhs), 32 * FR_WARPS, 0, s>>>(mk<double>(h), tab<double>(), fg,
+        x, b, r, zero_c, h.ndof, pstride(h, -1));
+  } else {
+    k_residual<DD, K, double><<<dim3(blocks(h.ndof, 256), nrhs), 256, 0, s>>>(mk<double>(h), plans<double>(h), x, b,
+        r, zero_c, h.ndof, pstride(h, -1));
+  }
+}
+template <int DD>
+int64_t residual_norm64(const HostLevel& h, const double* x, const double* b, double* r, double* partial, cudaStream_t s) {
+  if constexpr (DD == 2) {
+    const FactRowGrid fg = fact_row_grid<K>(h.n);
+    k_fact_residual_norm<DD, K><<<(unsigned)fg.first[3], 32 * FR_WARPS, 0, s>>>(mk<double>(h), tab<double>(), fg, x,
+        b, r, partial);
+    return fg.first[3];
+  } else {
+    const int64_t nb = residual_norm_blocks(h.ndof);
+    k_residual_norm_rp<DD, K, double><<<(unsigned)nb, RN_THREADS, 0, s>>>(mk<double>(h), plans<double>(h), x, b, r,
+        partial);
+    return nb;
   }
 }
 
 void apply(const HostLevel& h, int f32, const void* x, void* y, int nrhs, cudaStream_t s) {
-  const dim3 grid(blocks(h.ndof, 256), nrhs);
   if (f32)
-    k_apply<D, K, float><<<grid, 256, 0, s>>>(mk<float>(h), plans<float>(h), (const float*)x, (float*)y, h.ndof);
-  else if constexpr (D == 2)
-    fact_apply(h, (const double*)x, nullptr, (double*)y, 0, nrhs, ProbStride{}, s);
+    k_apply<D, K, float><<<dim3(blocks(h.ndof, 256), nrhs), 256, 0, s>>>(mk<float>(h), plans<float>(h), (const float*)x,
+                                                                        (float*)y, h.ndof);
   else
-    k_apply<D, K, double><<<grid, 256, 0, s>>>(mk<double>(h), plans<double>(h), (const double*)x, (double*)y,
-                                               h.ndof);
+    apply64<D>(h, (const double*)x, (double*)y, nrhs, s);
 }
 
 void residual(const HostLevel& h, int f32, const void* x, const void* b, void* r, int zero_c, int nrhs,
               cudaStream_t s) {
-  const dim3 grid(blocks(h.ndof, 256), nrhs);
   if (f32)
-    k_residual<D, K, float><<<grid, 256, 0, s>>>(mk<float>(h), plans<float>(h), (const float*)x, (const float*)b,
-                                                 (float*)r, zero_c, h.ndof, pstride(h, -1));
-  else if constexpr (D == 2)
-    fact_apply(h, (const double*)x, (const double*)b, (double*)r, zero_c, nrhs, pstride(h, -1), s);
+    k_residual<D, K, float><<<dim3(blocks(h.ndof, 256), nrhs), 256, 0, s>>>(mk<float>(h), plans<float>(h),
+        (const float*)x, (const float*)b, (float*)r, zero_c, h.ndof, pstride(h, -1));
   else
-    k_residual<D, K, double><<<grid, 256, 0, s>>>(mk<double>(h), plans<double>(h), (const double*)x,
-                                                  (const double*)b, (double*)r, zero_c, h.ndof, pstride(h, -1));
+    residual64<D>(h, (const double*)x, (const double*)b, (double*)r, zero_c, nrhs, s);
 }
 
 void restrict_(const HostLevel& f, const HostLevel& c, int f32, const void* rf, void* bc, int nrhs, cudaStream_t s) {
@@ -1053,32 +1075,30 @@ int64_t residual_norm_count(const HostLevel& h) {
 
 int64_t residual_norm(const HostLevel& h, const double* x, const double* b, double* r, double* partial,
                       cudaStream_t s) {
-  const int64_t nb = residual_norm_count(h);
-  if constexpr (D == 2)
-    k_fact_residual_norm<D, K><<<(unsigned)nb, 32 * FR_WARPS, 0, s>>>(mk<double>(h), tab<double>(), fact_row_grid<K>(h.n), x, b,
-                                                                  r, partial);
-  else
-    k_residual_norm_rp<D, K, double><<<(unsigned)nb, RN_THREADS, 0, s>>>(mk<double>(h), plans<double>(h), x, b, r,
-                                                                         partial);
-  return nb;
+  return residual_norm64<D>(h, x, b, r, partial, s);
 }
 
 void load_vector(const HostLevel& h, const double* f, const double* g, double* b, cudaStream_t s) {
   k_load<D, K><<<blocks(h.ndof, 256), 256, 0, s>>>(mk<double>(h), tab<double>(), f, g, b);
 }
 
-__global__ void k_copy_constrained(const Lvl<D, K, double> L, const double* __restrict__ r, double* __restrict__ z) {
+// The V-cycle's result as FP64: z = the level vector X, on constrained rows r
+// (vector blockIdx.y of several, ndof apart).
+template <typename T>
+__global__ void __launch_bounds__(256) k_result(const Lvl<D, K, double> L, const T* X, const double* r, double* z) {
+  pdl_wait();
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= L.ndof) return;
-  r += blockIdx.y * L.ndof;   // vector blockIdx.y of nvec, ndof apart
-  z += blockIdx.y * L.ndof;
+  const int64_t q = blockIdx.y * L.ndof + g;
   int idx[D];
-  const int comp = decode(L, g, idx);
-  if (is_constrained(L, comp, idx)) z[g] = r[g];
+  const int comp = decode32(L, (int)g, idx);
+  z[q] = is_constrained(L, comp, idx) ? r[q] : (double)X[q];
 }
 
-void copy_constrained(const HostLevel& h, const double* r, double* z, int nvec, cudaStream_t s) {
-  k_copy_constrained<<<dim3(blocks(h.ndof, 256), nvec), 256, 0, s>>>(mk<double>(h), r, z);
+void result(const HostLevel& h, int f32, const void* X, const double* r, double* z, int nvec, cudaStream_t s) {
+  const dim3 grid(blocks(h.ndof, 256), nvec);
+  if (f32) launch_pdl(k_result<float>, grid, 256, 0, s, mk<double>(h), (const float*)X, r, z);
+  else launch_pdl(k_result<double>, grid, 256, 0, s, mk<double>(h), (const double*)X, r, z);
 }
 
 DKOps make_ops() {
@@ -1101,7 +1121,7 @@ DKOps make_ops() {
   o.line_sweep = line_sweep;
   o.line_fits = line_fits;
   o.coarse_assemble = coarse_assemble;
-  o.copy_constrained = copy_constrained;
+  o.result = result;
   o.residual_norm = residual_norm;
   o.residual_norm_count = residual_norm_count;
   o.load_vector = load_vector;

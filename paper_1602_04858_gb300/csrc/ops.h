@@ -167,7 +167,8 @@ struct DKOps {
   // load vector of cellwise-constant f (D x ncell) and g (ncell, may be null), FP64
   void (*load_vector)(const HostLevel&, const double* f, const double* g, double* b, cudaStream_t);
   // z[g] = r[g] on the constrained dofs (FP64), nvec vectors ndof apart
-  void (*copy_constrained)(const HostLevel&, const double* r, double* z, int nvec, cudaStream_t);
+  // z = X (of the handle's type) as FP64, on constrained rows r
+  void (*result)(const HostLevel&, int f32, const void* X, const double* r, double* z, int nvec, cudaStream_t);
 };
 
 // Records msg as the text of mg_last_error() and returns s.
