@@ -248,6 +248,10 @@ def aggregate_throughput(dofs, steps, local_ms, dist=None, device="cpu"):
 
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of
+# DRAM bytes of an average launch of the finest level's line sweeps, by workload
+# (profiles/line_sweep_channels256_fp32.md: two launches of three passes to one of five)
+LINE_SWEEP_DRAM_BYTES = {"channels_256": (2 * 146.2e6 + 165.3e6) / 3}
+
 # the FP32 colour pass on the finest level of a workload, by workload and
 # kernel, from an ncu capture of the kernel as it stands; each has to be taken
 # again whenever its kernel changes (a workload without an entry reports null).
@@ -538,29 +542,29 @@ def main():
         clocks["window"] = "0.6 s of untimed V-cycles, then the timed region"
     value, ms_max = aggregate_throughput(N, args.steps, ms, dist, dev)
 
-    # --- dominant kernel: finest-level colour pass ---------------------------------
-    # In the V-cycle the 2C - 1 passes of a symmetric smoothing step run back to
-    # back (programmatic dependent launch overlaps each pass's prologue with
-    # the previous pass), so the average launch duration is taken over whole
-    # steps: CUDA events on the launching stream around each step of 2C - 1 passes.
-    # Events around every single pass break that overlap; that (pessimistic)
-    # figure is reported beside it as isolated_launch_ms.
+    # --- dominant kernel: the finest level's smoothing --------------------------------
+    # The smoother runs the passes of one class of vertex lines in one launch (up to
+    # five: mg_time_passes times two symmetric steps as the V-cycle runs them, per
+    # pass).  Bytes: each launch streams the inverses of its colours once, each pass
+    # its vectors.  The time of single colour passes, one launch each with events
+    # around it, is reported beside it as isolated_launch_ms.
     J = w["n_levels"] - 1
     C = 3 ** w["d"]
     order = list(range(C)) + list(range(C - 2, -1, -1))
-    step_bytes = sum(colour_pass_bytes(*G.patch_info(J, col), 4, 4) for col in order)
+    runs = []
+    for col in order + order[1:]:   # two steps; consecutive passes of a class, at most five
+        if not runs or runs[-1][-1] // 3 != col // 3 or len(runs[-1]) == 5:
+            runs.append([])
+        runs[-1].append(col)
+    run_passes = sum(len(q) for q in runs)
+    step_bytes = 0
+    for q in runs:
+        for i, col in enumerate(q):
+            npatch, nv = G.patch_info(J, col)
+            step_bytes += colour_pass_bytes(npatch, nv, 4, 4)
+            if col in q[:i]:
+                step_bytes -= npatch * nv * nv * 4
     G.level_load(J, torch.zeros_like(r), r)
-    reps = max(4, args.steps // 2)
-    steps_ev = []
-    for rep in range(reps + 1):
-        a = torch.cuda.Event(enable_timing=True)
-        b = torch.cuda.Event(enable_timing=True)
-        a.record(stream)
-        for col in order:
-            G.colour_pass(J, col)
-        b.record(stream)
-        if rep > 0:
-            steps_ev.append((a, b))
     iso = []
     for col in order:
         a = torch.cuda.Event(enable_timing=True)
@@ -570,12 +574,11 @@ def main():
         b.record(stream)
         iso.append((a, b))
     torch.cuda.synchronize()
-    tot_ms = sum(a.elapsed_time(b) for a, b in steps_ev)
-    npasses = len(order) * len(steps_ev)
     hbm, peak_kind = peaks()
-    achieved = step_bytes * len(steps_ev) / (tot_ms / 1e3) / 1e9
-    avg_launch_ms = tot_ms / npasses
-    per_launch_bytes = step_bytes / len(order)
+    pass_us = min(G.time_passes(J) for _ in range(3))
+    achieved = step_bytes / run_passes / (pass_us / 1e6) / 1e9
+    avg_launch_ms = pass_us * run_passes / len(runs) / 1e3
+    per_launch_bytes = step_bytes / len(runs)
     isolated_launch_ms = sum(a.elapsed_time(b) for a, b in iso) / len(iso)
 
     # --- where the V-cycle's time goes: per level, the pass time (graph of two
@@ -590,7 +593,7 @@ def main():
         C = 3 ** w["d"]
         passes = 2 * ((2 * C - 1) + (2 * C - 2) * (m - 1))
         us = G.time_passes(j)
-        level_breakdown[str(j)] = {"n": w["n_coarse"] << j, "kernel": pass_kernels[j], "us_per_pass": us,
+        level_breakdown[str(j)] = {"n": w["n_coarse"] << j, "kernel": "line sweep", "us_per_pass": us,
                                    "passes_per_vcycle": passes, "ms_per_vcycle": us * passes / 1e3}
 
     # --- companions: FP64 and BF16-inverse V-cycles, time to 1e-8 ----------------
@@ -690,14 +693,12 @@ def main():
                 "gpu_launches": int(launches),
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                              "frac": achieved / hbm,
-                             "traffic": FINEST_PASS_DRAM_BYTES.get((WORKLOAD, pass_kernels[J])),
-                             "kernel": {"warp": "k_colour_pass", "block": "k_colour_pass_cta",
-                                        "persistent blocks": "k_colour_pass_ctap"}[pass_kernels[J].split(" (")[0]]
-                                       + "<%d,%d,float,float> (finest level)" % (w["d"], w["degree"]),
+                             "traffic": LINE_SWEEP_DRAM_BYTES.get(WORKLOAD),
+                             "kernel": "k_line_sweep<%d,%d,float,float> (finest level)" % (w["d"], w["degree"]),
                              "peak_kind": peak_kind, "avg_launch_ms": avg_launch_ms,
                              "bytes_per_launch": per_launch_bytes, "isolated_launch_ms": isolated_launch_ms,
-                             "timing": f"CUDA events around back-to-back symmetric steps ({len(order)} passes) on the "
-                                       "launching stream, as the passes run inside the V-cycle"},
+                             "timing": f"two symmetric steps ({run_passes} passes in {len(runs)} launches) replayed as a "
+                                       "CUDA graph, as the passes run inside the V-cycle"},
                 "clocks": clocks,
                 "roofline_vcycle": {"model": "algorithmic bytes of one V-cycle: per level the patch inverses once "
                                              "if the level's set fits the L2 cache, else once per sweep, plus the "
