@@ -1141,12 +1141,14 @@ mg_status mg_level_load(mg_handle* h, int level, const double* x, const double* 
   if ((x && !is_device_ptr(x)) || (b && !is_device_ptr(b)))
     return fail(MG_ERR_INVALID_ARG, "x and b must be device pointers");
   HostLevel& L = h->lv[level];
+  // b first: a line sweep reads b before it waits for the launch ahead of it, which in
+  // mg_smooth is then the one that writes x (in the V-cycle a memset or the prolongation)
   if (h->prec == P64) {
-    if (x) CU(cudaMemcpyAsync(L.X, x, L.ndof * 8, cudaMemcpyDeviceToDevice, h->stream));
     if (b) CU(cudaMemcpyAsync(L.B, b, L.ndof * 8, cudaMemcpyDeviceToDevice, h->stream));
+    if (x) CU(cudaMemcpyAsync(L.X, x, L.ndof * 8, cudaMemcpyDeviceToDevice, h->stream));
   } else {
-    if (x) { launch_d2f(x, (float*)L.X, L.ndof, h->stream); ++h->launches; }
     if (b) { launch_d2f(b, (float*)L.B, L.ndof, h->stream); ++h->launches; }
+    if (x) { launch_d2f(x, (float*)L.X, L.ndof, h->stream); ++h->launches; }
   }
   CU(cudaGetLastError());
   return MG_OK;

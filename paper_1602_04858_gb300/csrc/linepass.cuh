@@ -984,7 +984,8 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
   }
   __syncthreads();   // rows, barriers, end coefficients
   if (A.cl > 1) cluster_arrive();   // barriers ready
-  // b and c strips: columns of cells va - 2 .. vb
+  // b and c strips: columns of cells va - 2 .. vb, read ahead of the wait: the launch
+  // before writes x only, and what wrote b ended before that one began
   const int wc = m + 3, x0 = (va - 2) * K1;
   const int wx = wc * K1 + 1;
   const uint32_t wmag = 0xffffffffu / (uint32_t)wx + 1u;   // e / wx as the high word of e wmag, for e below 2^32 / wx
