@@ -31,7 +31,11 @@
 //   2. delta = S_v r: lane (row group g, part s) takes the columns s, s + SPL,
 //      ...; FP32: the parts are reduced and scattered by shuffles so that lane l
 //      ends with row l; elsewhere through shared memory, FP64 with groups of
-//      rows that keep more lanes on its units;
+//      rows that keep more lanes on its units.  Every warp of a team reads the
+//      whole r, and on the shuffle path nothing orders the team's warps after
+//      that: the residuals of a team of several warps take turns in two buffers,
+//      so that the one a warp writes for the next patch is not the one a slower
+//      warp still reads, and the barrier of that next patch orders the one after;
 //   3. x|_v += delta in the strip.
 //
 // A warp beside the teams streams the inverses: it refills a buffer as soon as
@@ -249,9 +253,11 @@ struct LineShape {
   // the copies: shared-memory wavefronts, or the FP64 units (two FMAs per clock)
   static constexpr int WORK = sizeof(T) == 8 ? 16 * TW * NR * (NS + JCH * PR + 10)
                                              : TW * (NS * (NR == 1 ? 7 : 16) / 4 + JCH * (RG * (int)sizeof(TS) / 4 + 1) + 20 * NR);
-  // scratch per patch (T): residual ((r, r) pairs with one FP32 right-hand side), FP64 partial sums
+  // scratch per patch (T): residual ((r, r) pairs with one FP32 right-hand side), twice where
+  // only one barrier an item orders several warps; FP64 partial sums
   static constexpr int RP = (sizeof(T) == 4 && NR == 1) ? 2 : NR;
-  static constexpr int O_D = (NV * RP + 3) / 4 * 4;
+  static constexpr int RVS = (NV * RP + 3) / 4 * 4, RVN = SHF && TW > 1 ? 2 : 1;
+  static constexpr int O_D = RVN * RVS;
   static constexpr int SCR = O_D + (SHF ? 0 : (SPL * LPP * PR * NR + 3) / 4 * 4);
   static constexpr int S_BYTES = (int)(SL::STRIDE * sizeof(TS)), SC_BYTES = BF ? NVP * 4 : 0;
   static constexpr int BUF = ((GPW * (S_BYTES + SC_BYTES) + 127) / 128) * 128;   // one inverse buffer
@@ -906,7 +912,8 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
   v[0] = 2;
   v[1] = A.first[0] + 3 * (D == 2 ? line : line % A.cnt[0]);
   if (D == 3) v[D - 1] = A.first[1] + 3 * (line / A.cnt[0]);
-  T* rv = reinterpret_cast<T*>(smem + lay.scr) + (team * GPW + g) * C::SCR;
+  T* const scr = reinterpret_cast<T*>(smem + lay.scr) + (team * GPW + g) * C::SCR;
+  T* rv = scr;   // residual buffer of the current item
   unsigned char* bufs = smem + lay.buf + team * A.nsb * C::BUF;
   full += team * A.nsb;
   empty += team * A.nsb;
@@ -1209,7 +1216,7 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
           }
         }
         if constexpr (!C::SHF) {
-          T* dp = rv + C::O_D + (part * (LPP * PR) + grp * PR) * NR;
+          T* dp = scr + C::O_D + (part * (LPP * PR) + grp * PR) * NR;
           if constexpr (NR == 1 && sizeof(T) == 4) {
 #pragma unroll
             for (int i = 0; i < PR; i += 4) *reinterpret_cast<float4*>(dp + i) = make_float4(d[i][0], d[i + 1][0], d[i + 2][0], d[i + 3][0]);
@@ -1253,7 +1260,7 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
 #pragma unroll
           for (int rr = 0; rr < NR; ++rr) delta[rr] = d[0][rr];
         } else {
-          const T* dp = rv + C::O_D + (lp + it * LW) * NR;
+          const T* dp = scr + C::O_D + (lp + it * LW) * NR;
           ld_rhs<T, NR>(dp, delta);
 #pragma unroll
           for (int q2 = 1; q2 < SPL; ++q2) {
@@ -1299,6 +1306,7 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
         sb = 0;
         phase ^= 1u;
       }
+      if constexpr (C::RVN == 2) rv = rv == scr ? scr + C::RVS : scr;
     }
     // the next pass reads what this one wrote: the block's teams, then the
     // neighbour blocks
