@@ -226,6 +226,9 @@ mg_status mg_sync(mg_handle* h);
  * [0, 60] s allowed).  On expiry a kernel records MG_ERR_DEVICE_TIMEOUT for
  * mg_sync / mg_solve, waits (bounded) for its own copies in flight and
  * returns early: no trap, no hang; the output of that call is incomplete.
+ * (The blocks of a line sweep also wait for one another's updates: at most for
+ * what the neighbours' own waits within the limit may add up to in that
+ * launch, and a second.)
  * A limit of 0 makes every wait report a timeout at once, which is how the
  * error path is tested.  Synchronises the stream; the captured V-cycle is
  * rebuilt on its next use. */

@@ -705,6 +705,7 @@ void line_sweep_nr(const HostLevel& h, int cross, int ns, const int* cx, void* x
   a.pc = sp.pc;
   a.teams = sp.teams;
   a.nsb = sp.nsb;
+  a.nb_ns = line_neighbour_limit(h.wait_ns, ns, (h.n - 1 + sp.cl - 1) / sp.cl, sp.teams, C::GPW);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(a.nlines * sp.cl), groups);
   cfg.blockDim = dim3(C::TT * sp.teams + 32);

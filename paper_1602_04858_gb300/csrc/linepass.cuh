@@ -669,7 +669,24 @@ struct LineArgs {
   const void* S[3];      // inverses of the class's colours by x digit
   int64_t s_prob[3];     // bytes between problems of a group
   int nlo, nhi;          // patch rows in the patch's lower and upper cell along x
+  uint64_t nb_ns;        // limit of the waits for the neighbour blocks (line_neighbour_limit)
 };
+
+// Limit of a block's wait for a neighbour's strip or updates (ns).  A block is at most
+// as far behind as its own waits, each within the handle's limit wait_ns, can hold up
+// the line: pass s of a block ends no later than its items of that pass take after the
+// later of its own and its neighbours' pass s - 1, so the waits of one block's items of
+// the whole run bound it, however they are spread over the line.  A second is left for
+// the work itself.  (A team that gives up ends the waits of its block, so that a copy
+// that never lands costs one wait a block, not one an item.)
+constexpr uint64_t line_neighbour_limit(uint64_t wait_ns, int passes, int vertices, int teams, int gpw) {
+  const int patches = (vertices + 2) / 3;   // of a block and pass
+  return wait_ns * (uint64_t)(passes * ((patches + teams * gpw - 1) / (teams * gpw))) + 1000000000ull;
+}
+static_assert(line_neighbour_limit(0, 5, 43, 6, 1) == 1000000000ull, "no wait but for the work");
+static_assert(line_neighbour_limit(2000000000ull, 1, 3, 8, 1) > 2000000000ull, "longer than one item's wait");
+static_assert(line_neighbour_limit(60000000000ull, 5, 43, 6, 1) > 5 * 3 * 60000000000ull, "15 patches on 6 teams, 5 passes");
+static_assert(line_neighbour_limit(60000000000ull, 5, 4095, 1, 1) > 5 * 1365 * 60000000000ull, "no overflow on the longest lines");
 
 // (relaxed: only mbarrier initialisations, fenced by mbar_init, are published;
 // a release would wait for every copy in flight)
@@ -687,8 +704,10 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Waits (at most limit_ns) for an arrival of another block of the cluster.
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
+// Waits (at most limit_ns, and no longer once *given_up has the bit 2) for an arrival of
+// another block of the cluster.
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, uint64_t limit_ns,
+                                                  const volatile int* given_up) {
   const uint32_t a = smem_u32(bar);
   uint64_t t0 = 0;
   for (;;) {
@@ -701,7 +720,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
     if (ok) return true;
     const uint64_t t = globaltimer_ns();
     if (t0 == 0) t0 = t;
-    else if (t - t0 > limit_ns) return false;
+    else if (t - t0 > limit_ns || (*given_up & 2)) return false;
   }
 }
 __device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank) {
@@ -775,7 +794,6 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
   constexpr int K1 = K + 1, NV = C::NV, LW = C::LW, GPW = C::GPW, NVP = C::NVP, SPL = C::SPL, PR = C::PR, LPP = C::LPP;
   constexpr int Z0 = C::Z0, ZP = C::ZP, ZM = C::ZM, NS = C::NS, NIT = C::NIT;
   constexpr int EB = NR * (int)sizeof(T);   // bytes of a strip entry (the right-hand sides together)
-  constexpr uint64_t NB_LIMIT = 4000000000ull;   // bound of the waits for the neighbour blocks (ns)
   extern __shared__ __align__(128) unsigned char smem[];
   pdl_launch_dependents();   // the next launch's blocks prepare beside this one's
   const int tid = threadIdx.x;
@@ -797,7 +815,7 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
   const int oends = ocs + R::CROWS * A.pc * (int)sizeof(T);   // coefficients of the line's first and last patch
   int* xrow = reinterpret_cast<int*>(smem + lay.rows);   // flat index of x node 0 per x row (-1: outside)
   int* brow = xrow + R::XROWS;
-  volatile int* quit = brow + 2 * R::BROWS;   // a team gave up waiting
+  volatile int* quit = brow + 2 * R::BROWS;   // 1: a team gave up waiting, 2: a wait for a neighbour ran out
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + lay.bars);   // copies landed [team][buffer]
   uint64_t* empty = full + A.teams * A.nsb;                        // buffers free
   // neighbour blocks [left, right]: strip loaded, then its updates of pass s
@@ -894,7 +912,7 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
         did = true;
       }
       if (__any_sync(0xffffffffu, did)) t0 = globaltimer_ns();
-      else if (*quit || globaltimer_ns() - t0 > wait_ns + NB_LIMIT) break;
+      else if (*quit || globaltimer_ns() - t0 > wait_ns + A.nb_ns) break;
       else __nanosleep(20);
     }
     // no copy may land after the block has left: wait (bounded) for the last one
@@ -1048,11 +1066,24 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
   }
   cp_async_commit();
   const int ml = left_nb ? va - (1 + (rank - 1) * nx / A.cl) : 0;   // vertices of the block to the left
-  auto wait_nb = [&](int a) {   // a = 0: the neighbours' strips are loaded, s + 1: their updates of pass s are here
+  // a = 0: the neighbours' strips are loaded, s + 1: their updates of pass s are here
+  auto wait_nb = [&](int a) {
     bool ok = true;
-    if (left_nb) ok = mbar_wait_cluster(nbs + a, 0, NB_LIMIT);
-    if (right_nb) ok = mbar_wait_cluster(nbs + NBS + a, 0, NB_LIMIT) && ok;
-    if (!ok) atomicExch(err, 2);
+    if (left_nb) ok = mbar_wait_cluster(nbs + a, 0, A.nb_ns, quit);
+    if (right_nb) ok = mbar_wait_cluster(nbs + NBS + a, 0, A.nb_ns, quit) && ok;
+    if (!ok) {
+      atomicOr(const_cast<int*>(quit), 2);
+      atomicExch(err, 2);
+    }
+  };
+  // The inverses of an item: at most the handle's limit, and no longer once a team of
+  // the block has given up (the copying warp then stops refilling buffers)
+  auto wait_full = [&](uint64_t* bar, uint32_t parity) {
+    if (mbar_try_wait(bar, parity)) return true;
+    const uint64_t since = globaltimer_ns();
+    while (!mbar_try_wait(bar, parity))
+      if (*quit || globaltimer_ns() - since > wait_ns) return mbar_try_wait(bar, parity);
+    return true;
   };
   auto block_sync = [&]() {
     __syncwarp();
@@ -1145,7 +1176,7 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
       unsigned char* sbuf = bufs + sb * C::BUF;
       const float* scl = reinterpret_cast<const float*>(sbuf + GPW * C::S_BYTES) + g * NVP;
       // (bounded wait; BF16: the inverses' row scales enter r)
-      if constexpr (C::BF) ready = wait_ns != 0 && (ready || mbar_wait_bounded(full + sb, phase, wait_ns));
+      if constexpr (C::BF) ready = wait_ns != 0 && (ready || wait_full(full + sb, phase));
       auto put_r = [&](int row, int bofs, const T (&t)[NR]) {
         T r[NR];
         ld_rhs<T, NR>(at(bofs), r);
@@ -1161,11 +1192,11 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
       if constexpr (C::Z1 > 0) {
         if (rb >= 0) put_r(rb, bp, t1);
       }
-      if constexpr (!C::BF) ready = wait_ns != 0 && (ready || mbar_wait_bounded(full + sb, phase, wait_ns));
+      if constexpr (!C::BF) ready = wait_ns != 0 && (ready || wait_full(full + sb, phase));
       if (team_sync_or<C::TW>(team, !ready)) {
         if (tl == 0) {
           atomicExch(err, 2);
-          *quit = 1;
+          atomicOr(const_cast<int*>(quit), 1);
         }
         return false;
       }
@@ -1316,6 +1347,23 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
   }
   // (everything the neighbours send has arrived: the word of a strip loaded too)
   if (A.cl > 1) wait_nb(0);
+  // A block leaves once everything its neighbours send has landed.  Where a wait for it
+  // ran out they may be slower still, and a store into a block that has left would be a
+  // fault: the block then stays until every other one of the line has left or waits here
+  // too (all their waits are bounded), and until what they sent has landed.  (256^2 RT_1
+  // cycle: 1,486 us, 1,478 without; a barrier at the end of every block takes 1 % more,
+  // this test behind the stores 3 %.)
+  if (A.cl > 1) {
+    __syncwarp();
+    if (__any_sync(0xffffffffu, *quit & 2)) {
+      cluster_arrive();
+      cluster_wait();
+      for (int a = 0; a <= A.ns; ++a) {
+        if (left_nb) mbar_wait_bounded(nbs + a, 0, 100000000ull);
+        if (right_nb) mbar_wait_bounded(nbs + NBS + a, 0, 100000000ull);
+      }
+    }
+  }
   // (4) the updated rows of this segment's cells: va - 1 .. vb - 2, the first
   // and last block to the ends of the line
   const int lo = (va - 1) * K1, hi = rank == A.cl - 1 ? L.N : (vb - 1) * K1;
