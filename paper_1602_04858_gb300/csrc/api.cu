@@ -258,24 +258,29 @@ mg_status smooth_steps(mg_handle* h, int j, void* x, const void* b, void* acc, i
   }
   if (line_sweeps(h, j)) {
     // runs of passes whose colours differ in the x digit only: one launch each
+    // (a launch that fails ends the call: a V-cycle captured without it would be replayed)
     int cross = -1, ns = 0, cx[LINE_RUN];
     auto flush = [&]() {
       if (ns > 0) {
-        h->ops->line_sweep(L, cross, ns, cx, L.sprec, x, b, h->d_fail, nrhs, stream);
+        const cudaError_t e = h->ops->line_sweep(L, cross, ns, cx, L.sprec, x, b, h->d_fail, nrhs, stream);
+        if (e != cudaSuccess) {
+          cudaGetLastError();
+          return fail(MG_ERR_CUDA, std::string("line sweep: ") + cudaGetErrorString(e));
+        }
         ++h->launches;
       }
       ns = 0;
+      return MG_OK;
     };
     for (int s = 0; s < steps; ++s)
       for (int t = (s > 0 ? 1 : 0); t < 2 * C - 1; ++t) {
         const int col = t < C ? t : 2 * C - 2 - t;
         if (L.count[col] == 0) continue;
-        if (col / 3 != cross || ns == LINE_RUN) flush();
+        if (col / 3 != cross || ns == LINE_RUN) TRY(flush());
         cross = col / 3;
         cx[ns++] = col % 3;
       }
-    flush();
-    return MG_OK;
+    return flush();
   }
   for (int s = 0; s < steps; ++s) {
     for (int t = (s > 0 ? 1 : 0); t < 2 * C - 1; ++t) {

@@ -650,22 +650,25 @@ LineSplit line_split(const HostLevel& h, int groups) {
   int64_t lines = groups;   // of the largest class
   for (int e = 1; e < D; ++e) lines *= (nx + 2) / 3;
   // the launches of a hierarchy repeat: each thread keeps its last few answers
-  struct Memo { int n = 0, sms = 0; int64_t lines = 0; LineSplit q = {}; };
+  // (a device each: its registers, occupancy and SMs are its own)
+  struct Memo { int n = 0, dev = 0; int64_t lines = 0; LineSplit q = {}; };
   static thread_local Memo memo[16];
   static thread_local int next = 0;
+  int dev = 0;
+  cudaGetDevice(&dev);
   for (const Memo& m : memo)
-    if (m.n == h.n && m.lines == lines && m.sms == sms) return m.q;
+    if (m.n == h.n && m.lines == lines && m.dev == dev) return m.q;
   LineSplit best = {};
   line_split_form<T, TS, NR, 1>(nx, sms, lines, best);
   if constexpr (LineShape<D, K, T, TS, NR>::LEAN) line_split_form<T, TS, NR, 2>(nx, sms, lines, best);
-  memo[next] = {h.n, sms, lines, best};
+  memo[next] = {h.n, dev, lines, best};
   next = (next + 1) % 16;
   return best;   // cl = 0: no split fits the shared memory
 }
 
 template <typename T, typename TS, int NR>
-void line_sweep_nr(const HostLevel& h, int cross, int ns, const int* cx, void* x, const void* b, int* err,
-                   int groups, cudaStream_t s) {
+cudaError_t line_sweep_nr(const HostLevel& h, int cross, int ns, const int* cx, void* x, const void* b, int* err,
+                          int groups, cudaStream_t s) {
   using C = LineShape<D, K, T, TS, NR>;
   LineArgs a = {};
   int digit = cross;
@@ -677,7 +680,7 @@ void line_sweep_nr(const HostLevel& h, int cross, int ns, const int* cx, void* x
     a.cnt[e - 1] = colour_count(h.n, r);
     a.nlines *= a.cnt[e - 1];
   }
-  if (a.nlines == 0) return;
+  if (a.nlines == 0) return cudaSuccess;
   for (int c = 0; c < 3; ++c) {
     a.cntx[c] = colour_count(h.n, c);
     a.S[c] = h.S[c + 3 * cross];
@@ -722,27 +725,34 @@ void line_sweep_nr(const HostLevel& h, int cross, int ns, const int* cx, void* x
   cfg.numAttrs = sp.cl > 1 ? 2 : 1;
   const unsigned char* tabs = (const unsigned char*)h.R0 + line_tables_offset<T, TS>();
   auto launch = [&](auto kernel) {
-    cudaLaunchKernelEx(&cfg, kernel, mk<T>(h), a, tabs, (T*)x, (const T*)b, err, h.wait_ns, h.ndof, pstride(h, -1));
+    return cudaLaunchKernelEx(&cfg, kernel, mk<T>(h), a, tabs, (T*)x, (const T*)b, err, h.wait_ns, h.ndof, pstride(h, -1));
   };
   if constexpr (C::LEAN)
-    if (sp.mb == 2) return launch(k_line_sweep<D, K, T, TS, NR, 2>);
-  launch(k_line_sweep<D, K, T, TS, NR, 1>);
+    if (sp.mb == 2) {
+      line_attr<T, TS, NR, 2>();
+      return launch(k_line_sweep<D, K, T, TS, NR, 2>);
+    }
+  line_attr<T, TS, NR, 1>();
+  return launch(k_line_sweep<D, K, T, TS, NR, 1>);
 }
 
 template <typename T, typename TS>
-void line_sweep_t(const HostLevel& h, int cross, int ns, const int* cx, void* x, const void* b, int* err, int nrhs,
-                  cudaStream_t s) {
+cudaError_t line_sweep_t(const HostLevel& h, int cross, int ns, const int* cx, void* x, const void* b, int* err,
+                         int nrhs, cudaStream_t s) {
   const int g4 = (h.rhs_group < 4 || (h.rhs_prob > 0 && h.rhs_prob % 4 != 0)) ? 0 : nrhs / 4, rest = nrhs - 4 * g4;
   const size_t off = (size_t)4 * g4 * h.ndof;
-  if (g4 > 0) line_sweep_nr<T, TS, 4>(h, cross, ns, cx, x, b, err, g4, s);
-  if (rest > 0) line_sweep_nr<T, TS, 1>(h, cross, ns, cx, (T*)x + off, (const T*)b + off, err, rest, s);
+  cudaError_t e = cudaSuccess;
+  if (g4 > 0) e = line_sweep_nr<T, TS, 4>(h, cross, ns, cx, x, b, err, g4, s);
+  if (rest > 0 && e == cudaSuccess)
+    e = line_sweep_nr<T, TS, 1>(h, cross, ns, cx, (T*)x + off, (const T*)b + off, err, rest, s);
+  return e;
 }
 
-void line_sweep(const HostLevel& h, int cross, int ns, const int* cx, int prec, void* x, const void* b, int* err,
-                int nrhs, cudaStream_t s) {
-  if (prec == P64) line_sweep_t<double, double>(h, cross, ns, cx, x, b, err, nrhs, s);
-  else if (prec == P32) line_sweep_t<float, float>(h, cross, ns, cx, x, b, err, nrhs, s);
-  else line_sweep_t<float, __nv_bfloat16>(h, cross, ns, cx, x, b, err, nrhs, s);
+cudaError_t line_sweep(const HostLevel& h, int cross, int ns, const int* cx, int prec, void* x, const void* b,
+                       int* err, int nrhs, cudaStream_t s) {
+  if (prec == P64) return line_sweep_t<double, double>(h, cross, ns, cx, x, b, err, nrhs, s);
+  if (prec == P32) return line_sweep_t<float, float>(h, cross, ns, cx, x, b, err, nrhs, s);
+  return line_sweep_t<float, __nv_bfloat16>(h, cross, ns, cx, x, b, err, nrhs, s);
 }
 
 template <typename T, typename TS>

@@ -124,9 +124,9 @@ struct DKOps {
   void (*prolong_add)(const HostLevel& Lf, const HostLevel& Lc, int f32, const void* xc, void* xf, int nrhs,
                       cudaStream_t);
   // ns consecutive colour passes of the class of vertex lines `cross` (colour =
-  // x digit + 3 cross), x digits cx[0 .. ns), in one launch
-  void (*line_sweep)(const HostLevel&, int cross, int ns, const int* cx, int prec, void* x, const void* b, int* err,
-                     int nrhs, cudaStream_t);
+  // x digit + 3 cross), x digits cx[0 .. ns), in one launch; the launch's status
+  cudaError_t (*line_sweep)(const HostLevel&, int cross, int ns, const int* cx, int prec, void* x, const void* b,
+                            int* err, int nrhs, cudaStream_t);
   // whether the level's strips fit the line sweep's shared memory
   int (*line_fits)(const HostLevel&, int prec);
   // patch inverses of one colour into S (storage precision sprec); *fail set on a zero pivot

@@ -1,0 +1,74 @@
+"""Launches of the line sweeps on the host, with a stand-in for the CUDA runtime
+(fake_cudart.cpp: two devices, kernels do not run): the shared-memory limit is
+set on every device that a thread uses one after the other, whatever split it
+has worked out before, and a launch that fails is reported by the call and never
+becomes a replayed V-cycle without it.  The library's own objects are linked
+against the stand-in and run in a process of their own.
+"""
+import os
+import subprocess
+import sys
+
+import pytest
+
+from paper_1602_04858_gb300 import build as builder
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CUDA = os.path.dirname(os.path.dirname(builder.nvcc()))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    builder.build()
+    out = str(tmp_path_factory.mktemp("fake") / "libmgdarcy_fake.so")
+    objs = [os.path.join(builder.BUILD, o) for _, o, _ in builder.UNITS]
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I" + os.path.join(CUDA, "include"),
+                    os.path.join(HERE, "fake_cudart.cpp")] + objs + ["-o", out], check=True, capture_output=True)
+    return out
+
+
+def run(lib, body):
+    head = ("import ctypes, sys\nimport numpy as np\nfrom paper_1602_04858_gb300 import mgdarcy\n"
+            "L = mgdarcy.load(sys.argv[1])\n"
+            "L.fake_line_sweeps.restype = ctypes.c_long\n"
+            "def handle(precision='fp32', k=1, n0=4, levels=5, nrhs=1):\n"
+            "    n = n0 << (levels - 1)\n"
+            "    return mgdarcy.Multigrid(2, n0, levels, k, 0.01, np.ones(n * n), precision=precision, dense_level=0,\n"
+            "                             nrhs=nrhs, stream=0)\n")
+    r = subprocess.run([sys.executable, "-c", head + body, lib], cwd=os.path.dirname(HERE), capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("k,precision", [(0, "fp32"), (1, "fp32"), (1, "fp64"), (2, "fp32")])
+def test_each_device_gets_its_limit(lib, k, precision):
+    run(lib, f"""
+for d in (0, 1, 0):
+    L.fake_set_device(d)
+    before = L.fake_line_sweeps(d)
+    G = handle({precision!r}, {k})
+    r = np.zeros(G.ndof())
+    G.vcycle(r, np.zeros_like(r))
+    G.smooth(4, np.zeros_like(r), r)
+    assert L.fake_line_sweeps(d) > before, d
+    G.close()
+""")
+
+
+def test_failed_launch_is_reported_and_not_replayed(lib):
+    run(lib, """
+G = handle()
+r = np.zeros(G.ndof())
+z = np.zeros_like(r)
+for call in (lambda: G.vcycle(r, z), lambda: G.smooth(4, z, r)):
+    L.fake_fail_launches(b'k_line_sweep')
+    try:
+        call()
+        raise SystemExit('the failed launch was not reported')
+    except mgdarcy.MGError as e:
+        assert e.status == 3 and 'line sweep' in str(e), e
+    L.fake_fail_launches(b'')
+    before = L.fake_line_sweeps(0)
+    call()
+    assert L.fake_line_sweeps(0) > before, 'a cycle without its sweeps was replayed'
+""")
