@@ -1629,7 +1629,7 @@ bool same_shape(const mg_handle* a, const mg_handle* b) {
     return false;
   for (int j = 0; j <= a->J; ++j)
     if (a->lv[j].pass_cta != b->lv[j].pass_cta || a->lv[j].rhs_group != b->lv[j].rhs_group ||
-        a->lv[j].cta_tpr != b->lv[j].cta_tpr ||
+        a->lv[j].cta_tpr != b->lv[j].cta_tpr || a->lv[j].line != b->lv[j].line ||
         a->lv[j].sprec != b->lv[j].sprec)
       return false;
   return true;

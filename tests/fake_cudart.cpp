@@ -18,8 +18,9 @@ cudaError_t last = cudaSuccess;
 std::string failing;
 std::map<const void*, std::string> names;
 std::map<std::pair<const void*, int>, size_t> limits;
-std::map<int, long> ran;                    // line sweeps per device, replays included
-struct Graph { long sweeps = 0; };
+using Counts = std::map<std::string, long>;  // launches by kernel name
+std::map<int, Counts> ran;                   // of each device, replays included
+struct Graph { Counts launches; };
 Graph* capture = nullptr;
 struct Config { dim3 grid, block; size_t smem; cudaStream_t s; } pushed;
 cudaError_t err(cudaError_t e) { return e == cudaSuccess ? e : (last = e); }
@@ -28,10 +29,7 @@ cudaError_t launch(const void* f, size_t smem) {
   if (!failing.empty() && n.find(failing) != std::string::npos) return err(cudaErrorLaunchFailure);
   auto it = limits.find({f, device});
   if (smem > (it == limits.end() ? 48 * 1024 : it->second)) return err(cudaErrorInvalidValue);
-  if (n.find("k_line_sweep") != std::string::npos) {
-    if (capture) ++capture->sweeps;
-    else ++ran[device];
-  }
+  ++(capture ? capture->launches : ran[device])[n];
   return cudaSuccess;
 }
 }  // namespace
@@ -39,7 +37,12 @@ cudaError_t launch(const void* f, size_t smem) {
 extern "C" {
 void fake_set_device(int d) { device = d; }
 void fake_fail_launches(const char* part) { failing = part; }
-long fake_line_sweeps(int d) { return ran[d]; }
+long fake_launches(int d, const char* part) {
+  long n = 0;
+  for (const auto& k : ran[d])
+    if (k.first.find(part) != std::string::npos) n += k.second;
+  return n;
+}
 
 void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
 void __cudaRegisterFatBinaryEnd(void**) {}
@@ -85,7 +88,10 @@ cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { *g = (cudaGraph
 cudaError_t cudaGraphGetNodes(cudaGraph_t, cudaGraphNode_t*, size_t* n) { *n = 0; return cudaSuccess; }
 cudaError_t cudaGraphNodeGetType(cudaGraphNode_t, cudaGraphNodeType* t) { *t = cudaGraphNodeTypeKernel; return cudaSuccess; }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t g, unsigned long long) { *e = (cudaGraphExec_t)new Graph(*(Graph*)g); return cudaSuccess; }
-cudaError_t cudaGraphLaunch(cudaGraphExec_t e, cudaStream_t) { ran[device] += ((Graph*)e)->sweeps; return cudaSuccess; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t e, cudaStream_t) {
+  for (const auto& k : ((Graph*)e)->launches) ran[device][k.first] += k.second;
+  return cudaSuccess;
+}
 cudaError_t cudaGraphDestroy(cudaGraph_t g) { delete (Graph*)g; return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t e) { delete (Graph*)e; return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = nullptr; return cudaSuccess; }

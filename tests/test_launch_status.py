@@ -1,8 +1,9 @@
-"""Launches of the line sweeps on the host, with a stand-in for the CUDA runtime
+"""Launches of the smoother on the host, with a stand-in for the CUDA runtime
 (fake_cudart.cpp: two devices, kernels do not run): the shared-memory limit is
 set on every device that a thread uses one after the other, whatever split it
-has worked out before, and a launch that fails is reported by the call and never
-becomes a replayed V-cycle without it.  The library's own objects are linked
+has worked out before; a launch that fails is reported by the call and never
+becomes a replayed V-cycle without it; and every problem of a batch smooths as
+its own pass_kernel asks.  The library's own objects are linked
 against the stand-in and run in a process of their own.
 """
 import os
@@ -30,7 +31,8 @@ def lib(tmp_path_factory):
 def run(lib, body):
     head = ("import ctypes, sys\nimport numpy as np\nfrom paper_1602_04858_gb300 import mgdarcy\n"
             "L = mgdarcy.load(sys.argv[1])\n"
-            "L.fake_line_sweeps.restype = ctypes.c_long\n"
+            "L.fake_launches.restype = ctypes.c_long\n"
+            "def launches(part, d=0): return L.fake_launches(d, part)\n"
             "def handle(precision='fp32', k=1, n0=4, levels=5, nrhs=1):\n"
             "    n = n0 << (levels - 1)\n"
             "    return mgdarcy.Multigrid(2, n0, levels, k, 0.01, np.ones(n * n), precision=precision, dense_level=0,\n"
@@ -45,12 +47,12 @@ def test_each_device_gets_its_limit(lib, k, precision):
     run(lib, f"""
 for d in (0, 1, 0):
     L.fake_set_device(d)
-    before = L.fake_line_sweeps(d)
+    before = launches(b'k_line_sweep', d)
     G = handle({precision!r}, {k})
     r = np.zeros(G.ndof())
     G.vcycle(r, np.zeros_like(r))
     G.smooth(4, np.zeros_like(r), r)
-    assert L.fake_line_sweeps(d) > before, d
+    assert launches(b'k_line_sweep', d) > before, d
     G.close()
 """)
 
@@ -68,7 +70,30 @@ for call in (lambda: G.vcycle(r, z), lambda: G.smooth(4, z, r)):
     except mgdarcy.MGError as e:
         assert e.status == 3 and 'line sweep' in str(e), e
     L.fake_fail_launches(b'')
-    before = L.fake_line_sweeps(0)
+    before = launches(b'k_line_sweep')
     call()
-    assert L.fake_line_sweeps(0) > before, 'a cycle without its sweeps was replayed'
+    assert launches(b'k_line_sweep') > before, 'a cycle without its sweeps was replayed'
+""")
+
+
+def test_batch_members_smooth_as_asked(lib):
+    """A problem with a forced colour-pass kernel and one left to the library, whose
+    timed choice is the same kernel (every timing is equal here, so the first one
+    tried), in either order: one smooths by colour passes, the other by line sweeps."""
+    run(lib, """
+def count(kernels):
+    B = mgdarcy.Batch([dict(dim=2, n_coarse=4, n_levels=4, degree=1, mu=0.01, c=np.ones(32 * 32), precision='fp32',
+                            pass_kernel=k) for k in kernels], nrhs=1, stream=0)
+    r = np.zeros(B.total())
+    at = launches(b'k_line_sweep'), launches(b'k_colour_pass')
+    B.vcycle(r, np.zeros_like(r))
+    out = launches(b'k_line_sweep') - at[0], launches(b'k_colour_pass') - at[1]
+    del B
+    return out
+lines, none = count([0])
+none2, passes = count([1])
+assert lines > 0 and passes > 0 and none == none2 == 0
+assert count([0, 1]) == (lines, passes)
+assert count([1, 0]) == (lines, passes)
+assert count([0, 0]) == (lines, 0)      # the same choice: one group, one launch for both
 """)
