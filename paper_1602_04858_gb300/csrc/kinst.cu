@@ -739,7 +739,18 @@ cudaError_t line_sweep_nr(const HostLevel& h, int cross, int ns, const int* cx, 
 template <typename T, typename TS>
 cudaError_t line_sweep_t(const HostLevel& h, int cross, int ns, const int* cx, void* x, const void* b, int* err,
                          int nrhs, cudaStream_t s) {
-  const int g4 = (h.rhs_group < 4 || (h.rhs_prob > 0 && h.rhs_prob % 4 != 0)) ? 0 : nrhs / 4, rest = nrhs - 4 * g4;
+  // Groups of four right-hand sides share each inverse, or each is on its own, with four
+  // times the lines to spread over the SMs, whichever the splits' estimated times say
+  // (the colour passes' timed grouping is that of other kernels).  Small levels are
+  // faster on their own (16^2 RT_1, 4 right-hand sides: 1.37 against 1.99 us per pass,
+  // FP64 4.8 against 17), large ones in groups (128^2: 4.8 against 9.3).  The estimate
+  // flatters groups in FP64 and single vectors with BF16 inverses; with these factors
+  // its choice takes 1 % longer than the faster one on average over 130 levels and
+  // numbers of right-hand sides, and nowhere over 10 % longer than groups.
+  constexpr double own = sizeof(T) == 8 ? 1.1 : (sizeof(TS) == 2 ? 0.95 : 1.0);
+  int g4 = (h.rhs_prob > 0 && h.rhs_prob % 4 != 0) ? 0 : nrhs / 4;
+  if (g4 > 0 && line_split<T, TS, 1>(h, 4 * g4).t < own * line_split<T, TS, 4>(h, g4).t) g4 = 0;
+  const int rest = nrhs - 4 * g4;
   const size_t off = (size_t)4 * g4 * h.ndof;
   cudaError_t e = cudaSuccess;
   if (g4 > 0) e = line_sweep_nr<T, TS, 4>(h, cross, ns, cx, x, b, err, g4, s);

@@ -22,6 +22,7 @@ using Counts = std::map<std::string, long>;  // launches by kernel name
 std::map<int, Counts> ran;                   // of each device, replays included
 struct Graph { Counts launches; };
 Graph* capture = nullptr;
+float elapsed = 1000.f, faster = 0.f;
 struct Config { dim3 grid, block; size_t smem; cudaStream_t s; } pushed;
 cudaError_t err(cudaError_t e) { return e == cudaSuccess ? e : (last = e); }
 cudaError_t launch(const void* f, size_t smem) {
@@ -36,6 +37,7 @@ cudaError_t launch(const void* f, size_t smem) {
 
 extern "C" {
 void fake_set_device(int d) { device = d; }
+void fake_timings_fall(int on) { faster = on ? 1.f : 0.f; }   // every timing shorter than the one before
 void fake_fail_launches(const char* part) { failing = part; }
 long fake_launches(int d, const char* part) {
   long n = 0;
@@ -99,5 +101,5 @@ cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = nullptr; r
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 1.f; return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = elapsed -= faster; return cudaSuccess; }
 }

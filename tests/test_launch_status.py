@@ -2,8 +2,9 @@
 (fake_cudart.cpp: two devices, kernels do not run): the shared-memory limit is
 set on every device that a thread uses one after the other, whatever split it
 has worked out before; a launch that fails is reported by the call and never
-becomes a replayed V-cycle without it; and every problem of a batch smooths as
-its own pass_kernel asks.  The library's own objects are linked
+becomes a replayed V-cycle without it; every problem of a batch smooths as its
+own pass_kernel asks; and what the line sweeps launch does not depend on the
+timings of the colour passes.  The library's own objects are linked
 against the stand-in and run in a process of their own.
 """
 import os
@@ -96,4 +97,28 @@ assert lines > 0 and passes > 0 and none == none2 == 0
 assert count([0, 1]) == (lines, passes)
 assert count([1, 0]) == (lines, passes)
 assert count([0, 0]) == (lines, 0)      # the same choice: one group, one launch for both
+""")
+
+
+@pytest.mark.parametrize("k,precision,nrhs", [(0, "fp32", 4), (1, "fp32", 8), (1, "fp64", 4), (1, "fp32_bf16inv", 5)])
+def test_line_sweeps_do_not_follow_colour_pass_timings(lib, tmp_path, k, precision, nrhs):
+    """Timings that make the colour passes' first candidate the fastest (four right-hand
+    sides together) and their last one (each on its own): the same sweeps are launched."""
+    for fall in (0, 1):
+        run(lib, f"""
+L.fake_timings_fall({fall})
+G = handle({precision!r}, {k}, nrhs={nrhs})
+g = ctypes.c_int()
+L.mg_level_rhs_group(G.h, 2, ctypes.byref(g))
+assert g.value == (1 if {fall} else 4), g.value
+r = np.zeros({nrhs} * G.ndof())
+at = launches(b'k_line_sweep'), launches(b'Li4ELi1EEE'), launches(b'Li1ELi1EEE')
+G.vcycle(r, np.zeros_like(r))
+now = launches(b'k_line_sweep') - at[0], launches(b'Li4ELi1EEE') - at[1], launches(b'Li1ELi1EEE') - at[2]
+assert now[0] == now[1] + now[2] > 0, now
+path = {str(tmp_path / "launches")!r}
+if {fall}:
+    assert open(path).read() == repr(now), now
+else:
+    open(path, 'w').write(repr(now))
 """)
