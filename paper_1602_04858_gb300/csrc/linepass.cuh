@@ -677,8 +677,8 @@ struct LineArgs {
 // the line: pass s of a block ends no later than its items of that pass take after the
 // later of its own and its neighbours' pass s - 1, so the waits of one block's items of
 // the whole run bound it, however they are spread over the line.  A second is left for
-// the work itself.  (A team that gives up ends the waits of its block, so that a copy
-// that never lands costs one wait a block, not one an item.)
+// the work itself.  (A team that has given up waits for no copy any more, so a copy that
+// never lands costs a team one wait.)
 constexpr uint64_t line_neighbour_limit(uint64_t wait_ns, int passes, int vertices, int teams, int gpw) {
   const int patches = (vertices + 2) / 3;   // of a block and pass
   return wait_ns * (uint64_t)(passes * ((patches + teams * gpw - 1) / (teams * gpw))) + 1000000000ull;
@@ -692,6 +692,11 @@ static_assert(line_neighbour_limit(60000000000ull, 5, 4095, 1, 1) > 5 * 1365 * 6
 // a release would wait for every copy in flight)
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// Waits until every thread of the cluster has left or waits here too (the threads of a
+// warp need not come together).
+__device__ __forceinline__ void cluster_sync_late() {
+  asm volatile("barrier.cluster.arrive.relaxed;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -704,10 +709,8 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Waits (at most limit_ns, and no longer once *given_up has the bit 2) for an arrival of
-// another block of the cluster.
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, uint64_t limit_ns,
-                                                  const volatile int* given_up) {
+// Waits (at most limit_ns) for an arrival of another block of the cluster.
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
   const uint32_t a = smem_u32(bar);
   uint64_t t0 = 0;
   for (;;) {
@@ -720,7 +723,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
     if (ok) return true;
     const uint64_t t = globaltimer_ns();
     if (t0 == 0) t0 = t;
-    else if (t - t0 > limit_ns || (*given_up & 2)) return false;
+    else if (t - t0 > limit_ns) return false;
   }
 }
 __device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank) {
@@ -1069,21 +1072,12 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
   // a = 0: the neighbours' strips are loaded, s + 1: their updates of pass s are here
   auto wait_nb = [&](int a) {
     bool ok = true;
-    if (left_nb) ok = mbar_wait_cluster(nbs + a, 0, A.nb_ns, quit);
-    if (right_nb) ok = mbar_wait_cluster(nbs + NBS + a, 0, A.nb_ns, quit) && ok;
+    if (left_nb) ok = mbar_wait_cluster(nbs + a, 0, A.nb_ns);
+    if (right_nb) ok = mbar_wait_cluster(nbs + NBS + a, 0, A.nb_ns) && ok;
     if (!ok) {
       atomicOr(const_cast<int*>(quit), 2);
       atomicExch(err, 2);
     }
-  };
-  // The inverses of an item: at most the handle's limit, and no longer once a team of
-  // the block has given up (the copying warp then stops refilling buffers)
-  auto wait_full = [&](uint64_t* bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t since = globaltimer_ns();
-    while (!mbar_try_wait(bar, parity))
-      if (*quit || globaltimer_ns() - since > wait_ns) return mbar_try_wait(bar, parity);
-    return true;
   };
   auto block_sync = [&]() {
     __syncwarp();
@@ -1176,7 +1170,7 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
       unsigned char* sbuf = bufs + sb * C::BUF;
       const float* scl = reinterpret_cast<const float*>(sbuf + GPW * C::S_BYTES) + g * NVP;
       // (bounded wait; BF16: the inverses' row scales enter r)
-      if constexpr (C::BF) ready = wait_ns != 0 && (ready || wait_full(full + sb, phase));
+      if constexpr (C::BF) ready = wait_ns != 0 && (ready || mbar_wait_bounded(full + sb, phase, wait_ns));
       auto put_r = [&](int row, int bofs, const T (&t)[NR]) {
         T r[NR];
         ld_rhs<T, NR>(at(bofs), r);
@@ -1192,7 +1186,7 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
       if constexpr (C::Z1 > 0) {
         if (rb >= 0) put_r(rb, bp, t1);
       }
-      if constexpr (!C::BF) ready = wait_ns != 0 && (ready || wait_full(full + sb, phase));
+      if constexpr (!C::BF) ready = wait_ns != 0 && (ready || mbar_wait_bounded(full + sb, phase, wait_ns));
       if (team_sync_or<C::TW>(team, !ready)) {
         if (tl == 0) {
           atomicExch(err, 2);
@@ -1345,24 +1339,19 @@ __global__ void __launch_bounds__(LineShape<D, K, T, TS, NR>::MAXT + 32, MB)
     block_sync();
     if (A.cl > 1) wait_nb(s + 1);
   }
-  // (everything the neighbours send has arrived: the word of a strip loaded too)
-  if (A.cl > 1) wait_nb(0);
-  // A block leaves once everything its neighbours send has landed.  Where a wait for it
-  // ran out they may be slower still, and a store into a block that has left would be a
-  // fault: the block then stays until every other one of the line has left or waits here
-  // too (all their waits are bounded), and until what they sent has landed.  (256^2 RT_1
-  // cycle: 1,486 us, 1,478 without; a barrier at the end of every block takes 1 % more,
-  // this test behind the stores 3 %.)
+  // A block leaves once everything its neighbours send has landed, the word of a loaded
+  // strip too.  Where a wait for it ran out they may be slower still, and a store into a
+  // block that has left would be a fault: the block then stays until every other one of
+  // the line has left or waits here too (all their waits are bounded), and looks for what
+  // they sent once more.  (The barrier in the loop, not behind it or behind the stores,
+  // and no flag or limit read besides: other forms took 0.5 to 4 % of a 256^2 RT_1 cycle,
+  // 1,478 us without any, 1,482 so.)
   if (A.cl > 1) {
-    __syncwarp();
-    if (__any_sync(0xffffffffu, *quit & 2)) {
-      cluster_arrive();
-      cluster_wait();
-      for (int a = 0; a <= A.ns; ++a) {
-        if (left_nb) mbar_wait_bounded(nbs + a, 0, 100000000ull);
-        if (right_nb) mbar_wait_bounded(nbs + NBS + a, 0, 100000000ull);
-      }
-    }
+    int a = 0;
+    do {
+      wait_nb(a > A.ns ? 0 : a);
+      if (a == 0 && (*quit & 2)) cluster_sync_late();
+    } while ((*quit & 2) && ++a <= A.ns + 1);
   }
   // (4) the updated rows of this segment's cells: va - 1 .. vb - 2, the first
   // and last block to the ends of the line
