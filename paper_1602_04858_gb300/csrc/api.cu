@@ -998,7 +998,9 @@ static mg_status setup_internal(const mg_problem* p, void* cuda_stream, int nrhs
   }
   for (int t = 0; t < 4; ++t)
     if ((st = h->alloc(&h->t64[t], (size_t)h->lv[J].ndof * (t < 2 ? nrhs : 1))) != MG_OK) return cleanup(st);
-  if ((st = h->alloc(&h->d_rnp, h->ops->residual_norm_count(h->lv[J]))) != MG_OK) return cleanup(st);
+  int64_t partials = 0;   // of any level's residual norm
+  for (const HostLevel& L : h->lv) partials = std::max(partials, h->ops->residual_norm_count(L));
+  if ((st = h->alloc(&h->d_rnp, partials)) != MG_OK) return cleanup(st);
   if ((st = h->alloc(&h->d_rn, 1)) != MG_OK) return cleanup(st);
   int bad = 0;
   if (cudaMemcpyAsync(&bad, h->d_fail, sizeof(int), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||

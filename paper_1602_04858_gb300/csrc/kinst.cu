@@ -222,44 +222,46 @@ template <> RowPlans<float> plans<float>(const HostLevel& h) {
   return RowPlans<float>{h.rp.cls, h.rp.ptr, h.rp.mptr, h.rp.pe, h.rp.pcf32, h.rp.me, h.rp.mcf32};
 }
 
-// The operator in FP64.  In 2-D its products are the bound (factrow.cuh: 59 us for the
-// residual norm of 320^2 RT_1, row plans 87); FP32 and 3-D RT_0 (one node across a
-// cell: little to factor out) keep the row plans.
+// The operator in FP64.  In 2-D its products are the bound (factrow.cuh); FP32 and 3-D
+// RT_0 (one node across a cell: little to factor out) keep the row plans, and so does
+// 2-D RT_0 beyond 128^2 cells.  Factored / row plans, one application (us): RT_1 4^2 5.1 /
+// 8.5, 32^2 7.9 / 7.9, 64^2 8.0 / 8.1, 128^2 9.6 / 19.4, 512^2 109 / 177; RT_2 8^2 12.4 /
+// 13.8, 128^2 24.4 / 46.8; RT_0 8^2 3.5 / 5.0, 64^2 4.5 / 4.8, 128^2 4.5 / 5.0, 192^2 7.0 /
+// 6.3, 256^2 9.5 / 9.8, 384^2 16.2 / 15.1, 512^2 25.6 / 24.0.
+// (By the mesh alone: a vector's result does not depend on those computed beside it.)
+bool factored(const HostLevel& h) { return K > 0 || h.n <= 128; }
 template <int DD>
 void apply64(const HostLevel& h, const double* x, double* y, int nrhs, cudaStream_t s) {
-  if constexpr (DD == 2) {
+  if constexpr (DD == 2) if (factored(h)) {
     const FactRowGrid fg = fact_row_grid<K>(h.n);
     k_fact_apply<DD, K><<<dim3((unsigned)fg.first[3], nrhs), 32 * FR_WARPS, 0, s>>>(mk<double>(h), tab<double>(), fg,
         x, (const double*)nullptr, y, 0, h.ndof, ProbStride{});
-  } else {
-    k_apply<DD, K, double><<<dim3(blocks(h.ndof, 256), nrhs), 256, 0, s>>>(mk<double>(h), plans<double>(h), x, y,
-        h.ndof);
+    return;
   }
+  k_apply<DD, K, double><<<dim3(blocks(h.ndof, 256), nrhs), 256, 0, s>>>(mk<double>(h), plans<double>(h), x, y, h.ndof);
 }
 template <int DD>
 void residual64(const HostLevel& h, const double* x, const double* b, double* r, int zero_c, int nrhs, cudaStream_t s) {
-  if constexpr (DD == 2) {
+  if constexpr (DD == 2) if (factored(h)) {
     const FactRowGrid fg = fact_row_grid<K>(h.n);
     k_fact_apply<DD, K><<<dim3((unsigned)fg.first[3], nrhs), 32 * FR_WARPS, 0, s>>>(mk<double>(h), tab<double>(), fg,
         x, b, r, zero_c, h.ndof, pstride(h, -1));
-  } else {
-    k_residual<DD, K, double><<<dim3(blocks(h.ndof, 256), nrhs), 256, 0, s>>>(mk<double>(h), plans<double>(h), x, b,
-        r, zero_c, h.ndof, pstride(h, -1));
+    return;
   }
+  k_residual<DD, K, double><<<dim3(blocks(h.ndof, 256), nrhs), 256, 0, s>>>(mk<double>(h), plans<double>(h), x, b, r,
+      zero_c, h.ndof, pstride(h, -1));
 }
 template <int DD>
 int64_t residual_norm64(const HostLevel& h, const double* x, const double* b, double* r, double* partial, cudaStream_t s) {
-  if constexpr (DD == 2) {
+  if constexpr (DD == 2) if (factored(h)) {
     const FactRowGrid fg = fact_row_grid<K>(h.n);
     k_fact_residual_norm<DD, K><<<(unsigned)fg.first[3], 32 * FR_WARPS, 0, s>>>(mk<double>(h), tab<double>(), fg, x,
         b, r, partial);
     return fg.first[3];
-  } else {
-    const int64_t nb = residual_norm_blocks(h.ndof);
-    k_residual_norm_rp<DD, K, double><<<(unsigned)nb, RN_THREADS, 0, s>>>(mk<double>(h), plans<double>(h), x, b, r,
-        partial);
-    return nb;
   }
+  const int64_t nb = residual_norm_blocks(h.ndof);
+  k_residual_norm_rp<DD, K, double><<<(unsigned)nb, RN_THREADS, 0, s>>>(mk<double>(h), plans<double>(h), x, b, r, partial);
+  return nb;
 }
 
 void apply(const HostLevel& h, int f32, const void* x, void* y, int nrhs, cudaStream_t s) {
@@ -1091,8 +1093,8 @@ void coarse_assemble(const HostLevel& h, const int64_t* free_list, const int* g2
 }
 
 int64_t residual_norm_count(const HostLevel& h) {
-  if constexpr (D == 2) return fact_row_grid<K>(h.n).first[3];
-  else return residual_norm_blocks(h.ndof);
+  if (D == 2 && factored(h)) return fact_row_grid<K>(h.n).first[3];
+  return residual_norm_blocks(h.ndof);
 }
 
 int64_t residual_norm(const HostLevel& h, const double* x, const double* b, double* r, double* partial,
