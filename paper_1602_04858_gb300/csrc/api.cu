@@ -812,6 +812,9 @@ static mg_status setup_internal(const mg_problem* p, void* cuda_stream, int nrhs
     // the coarser levels keep FP32 inverses
     L.sprec = (h->prec == P32B && j < J) ? P32 : h->prec;
     if (j == 0) continue;
+    // the kernel choices left to the library smooth by line sweeps (line_sweeps)
+    L.line = (p->pass_kernel == 0 || p->pass_kernel == 4 || p->pass_kernel == 5) && p->additive == 0.0 &&
+             !p->boundary_patches && h->ops->line_fits(L, L.sprec);
     const size_t sb = (L.sprec == P64) ? 8 : (L.sprec == P32 ? 4 : 2);
     {
       int64_t np = 0;
@@ -859,10 +862,6 @@ static mg_status setup_internal(const mg_problem* p, void* cuda_stream, int nrhs
       }
     }
   }
-  // the kernel choices left to the library smooth by line sweeps
-  for (int j = 1; j <= J; ++j)
-    h->lv[j].line = (p->pass_kernel == 0 || p->pass_kernel == 4 || p->pass_kernel == 5) &&
-                    h->ops->line_fits(h->lv[j], h->lv[j].sprec);
   if ((st = tune_passes(h, p->pass_kernel, nrhs)) != MG_OK) return cleanup(st);
   h->main.nrhs = nrhs;
   h->nrhs = nrhs;

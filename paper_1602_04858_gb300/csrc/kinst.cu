@@ -806,7 +806,7 @@ int build_template_t(const HostLevel& h, void* tabs, cudaStream_t s, std::string
   if (!ok || !build_cta_tables<D, K, T, TS, 4>(mk<T>(h), tab<T>(), blob_4, msg) ||
       !build_cta_tables<D, K, T, TS, 2>(mk<T>(h), tab<T>(), blob_2, msg) ||
       !build_cta_tables<D, K, T, TS, 8>(mk<T>(h), tab<T>(), blob_8, msg) ||
-      !build_line_tables<D, K, T, TS>(mk<T>(h), tab<T>(), blob_l, msg)) {
+      (h.line && !build_line_tables<D, K, T, TS>(mk<T>(h), tab<T>(), blob_l, msg))) {
     if (why) *why = "colour-pass tables of the " + std::to_string(h.n) + "^" + std::to_string(D) + " level: " + msg;
     return 1;
   }
@@ -814,7 +814,7 @@ int build_template_t(const HostLevel& h, void* tabs, cudaStream_t s, std::string
   std::memcpy(blob.data() + cta_tables_offset<T, TS, 4>(), blob_4.data(), blob_4.size());
   std::memcpy(blob.data() + cta_tables_offset<T, TS, 2>(), blob_2.data(), blob_2.size());
   std::memcpy(blob.data() + cta_tables_offset<T, TS, 8>(), blob_8.data(), blob_8.size());
-  std::memcpy(blob.data() + line_tables_offset<T, TS>(), blob_l.data(), blob_l.size());
+  if (h.line) std::memcpy(blob.data() + line_tables_offset<T, TS>(), blob_l.data(), blob_l.size());
   if (cudaMemcpyAsync(tabs, blob.data(), blob.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     if (why) *why = "upload of the colour-pass tables failed";
@@ -823,7 +823,8 @@ int build_template_t(const HostLevel& h, void* tabs, cudaStream_t s, std::string
   return 0;
 }
 
-// Builds the colour-pass tables on the host and uploads them; nonzero (with
+// Builds the colour-pass tables on the host (the line sweep's only where the level uses
+// it: 3 to 15 ms of a set-up) and uploads them; nonzero (with
 // a reason) if the rows of a patch type do not fit the lane plan.
 int build_template(const HostLevel& h, int sprec, void* tabs, cudaStream_t s, std::string* why) {
   if (sprec == P64) return build_template_t<double, double>(h, tabs, s, why);
