@@ -764,7 +764,8 @@ cudaError_t line_sweep_t(const HostLevel& h, int cross, int ns, const int* cx, v
 
 cudaError_t line_sweep(const HostLevel& h, int cross, int ns, const int* cx, int prec, void* x, const void* b,
                        int* err, int nrhs, cudaStream_t s) {
-  if (prec == P64) return line_sweep_t<double, double>(h, cross, ns, cx, x, b, err, nrhs, s);
+  if constexpr (K < 2)   // (line_fits)
+    if (prec == P64) return line_sweep_t<double, double>(h, cross, ns, cx, x, b, err, nrhs, s);
   if (prec == P32) return line_sweep_t<float, float>(h, cross, ns, cx, x, b, err, nrhs, s);
   return line_sweep_t<float, __nv_bfloat16>(h, cross, ns, cx, x, b, err, nrhs, s);
 }
@@ -777,7 +778,10 @@ bool line_fits_t(const HostLevel& h) {
 int line_fits(const HostLevel& h, int prec) {
   // RT_2 in FP64 keeps the colour passes: its product has no lanes to spare and
   // one team per SM (26.5 against 22.7 us per pass on 64^2, 12.4 against 7.6 on 32^2)
-  if (prec == P64) return K < 2 && line_fits_t<double, double>(h);
+  if (prec == P64) {
+    if constexpr (K < 2) return line_fits_t<double, double>(h);
+    return 0;
+  }
   if (prec == P32) return line_fits_t<float, float>(h);
   return line_fits_t<float, __nv_bfloat16>(h);
 }
