@@ -247,13 +247,13 @@ def aggregate_throughput(dofs, steps, local_ms, dist=None, device="cpu"):
     return dofs * steps * world / (ms_max / 1e3), ms_max
 
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of
-# DRAM bytes of an average launch of the finest level's line sweeps, by workload
-# (profiles/line_sweep_channels256_fp32.md: two launches of three passes to one of five)
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of an average launch of
+# the finest level's line sweeps, by workload (profiles/line_sweep_channels256_fp32.md:
+# two launches of three passes to one of five)
 LINE_SWEEP_DRAM_BYTES = {"channels_256": (2 * 146.2e6 + 165.3e6) / 3}
 
-# the FP32 colour pass on the finest level of a workload, by workload and
-# kernel, from an ncu capture of the kernel as it stands; each has to be taken
+# The same of one launch of the FP32 colour pass on the finest level, where it smooths
+# by colour passes (--pass-kernel), by workload and kernel, from an ncu capture of the kernel as it stands; each has to be taken
 # again whenever its kernel changes (a workload without an entry reports null).
 FINEST_PASS_DRAM_BYTES = {("channels_256", "warp"): 51.033344e6 + 0.011776e6,
                           # 64^3 RT_0: 9,261 patches of 20 dofs per colour
@@ -292,6 +292,42 @@ def colour_pass_bytes(count, nv, s_inv, s_v):
     """Algorithmic bytes of one colour pass: each patch streams its n_v x n_v
     inverse once and reads b_v, x_v and writes x_v (3 n_v vector entries)."""
     return count * (nv * nv * s_inv + 3 * nv * s_v)
+
+
+def smoothing_runs(d, lines):
+    """The colour passes of two symmetric smoothing steps, launch by launch: one
+    each, or (line sweeps) consecutive passes of one class of vertex lines
+    together, at most five."""
+    C = 3 ** d
+    order = list(range(C)) + list(range(C - 2, -1, -1))
+    runs = []
+    for col in order + order[1:]:
+        if not lines or not runs or runs[-1][-1] // 3 != col // 3 or len(runs[-1]) == 5:
+            runs.append([])
+        runs[-1].append(col)
+    return runs
+
+
+def line_sweep_bytes(run, d, k, n, patches, nv, s_inv, s_v):
+    """Algorithmic bytes of one line sweep: the inverses of the run's colours once
+    each, and x read and written and b read once for the dofs of the class's lines
+    (the interiors of all patches of a line of vertices along x together).
+    patches: patches per colour."""
+    N, lines, digit = n * (k + 1), 1, run[0] // 3
+    for _ in range(d - 1):
+        r, digit = digit % 3, digit // 3
+        lines *= len(range(r if r > 0 else 3, n, 3))
+    across, own = 2 * (k + 1), 2 * k + 1   # nodes of a patch in a cross direction: a component's own has no faces
+    dofs = across ** (d - 1) * (N - 1) + (d - 1) * own * across ** (d - 2) * N + across ** (d - 1) * N
+    return sum(patches[col] for col in set(run)) * nv * nv * s_inv + 3 * lines * dofs * s_v
+
+
+def smooths_by_lines(G, level, x, b):
+    """Whether the handle smooths a level by line sweeps: by the launches of one step
+    (2 C - 1 passes; loads and the store of the vectors come to three at most)."""
+    before = G.launches()
+    G.smooth(level, x, b, steps=1)
+    return G.launches() - before < 2 * 3 ** G.dim - 1
 
 
 def end_to_end(args, make, rh, N, barrier, dist, dev, world):
@@ -543,27 +579,29 @@ def main():
     value, ms_max = aggregate_throughput(N, args.steps, ms, dist, dev)
 
     # --- dominant kernel: the finest level's smoothing --------------------------------
-    # The smoother runs the passes of one class of vertex lines in one launch (up to
-    # five: mg_time_passes times two symmetric steps as the V-cycle runs them, per
-    # pass).  Bytes: each launch streams the inverses of its colours once, each pass
-    # its vectors.  The time of single colour passes, one launch each with events
-    # around it, is reported beside it as isolated_launch_ms.
+    # By default the passes of one class of vertex lines run in one launch (line sweeps),
+    # with a forced --pass-kernel one launch each; mg_time_passes times two symmetric
+    # steps as the V-cycle runs them, per pass.  Bytes: each launch streams the inverses
+    # of its colours and its vectors once.  The time of single colour passes, one launch
+    # each with events around it, is reported beside it as isolated_launch_ms.
     J = w["n_levels"] - 1
     C = 3 ** w["d"]
     order = list(range(C)) + list(range(C - 2, -1, -1))
-    runs = []
-    for col in order + order[1:]:   # two steps; consecutive passes of a class, at most five
-        if not runs or runs[-1][-1] // 3 != col // 3 or len(runs[-1]) == 5:
-            runs.append([])
-        runs[-1].append(col)
+    by_lines = {}
+    for j in range(1, J + 1):
+        v = torch.zeros(sum(G.sizes(j)), dtype=torch.float64, device=dev)
+        by_lines[j] = smooths_by_lines(G, j, v, torch.zeros_like(v))
+    runs = smoothing_runs(w["d"], by_lines[J])
     run_passes = sum(len(q) for q in runs)
-    step_bytes = 0
-    for q in runs:
-        for i, col in enumerate(q):
-            npatch, nv = G.patch_info(J, col)
-            step_bytes += colour_pass_bytes(npatch, nv, 4, 4)
-            if col in q[:i]:
-                step_bytes -= npatch * nv * nv * 4
+    patches, nv = [G.patch_info(J, col)[0] for col in range(C)], G.patch_info(J, 0)[1]
+    if by_lines[J]:
+        step_bytes = sum(line_sweep_bytes(q, w["d"], w["degree"], w["n_coarse"] << J, patches, nv, 4, 4) for q in runs)
+        kernel, traffic = "k_line_sweep", LINE_SWEEP_DRAM_BYTES.get(WORKLOAD)
+    else:
+        step_bytes = sum(colour_pass_bytes(patches[q[0]], nv, 4, 4) for q in runs)
+        kernel = {"warp": "k_colour_pass", "block": "k_colour_pass_cta",
+                  "persistent blocks": "k_colour_pass_ctap"}[pass_kernels[J].split(" (")[0]]
+        traffic = FINEST_PASS_DRAM_BYTES.get((WORKLOAD, pass_kernels[J]))
     G.level_load(J, torch.zeros_like(r), r)
     iso = []
     for col in order:
@@ -593,7 +631,8 @@ def main():
         C = 3 ** w["d"]
         passes = 2 * ((2 * C - 1) + (2 * C - 2) * (m - 1))
         us = G.time_passes(j)
-        level_breakdown[str(j)] = {"n": w["n_coarse"] << j, "kernel": "line sweep", "us_per_pass": us,
+        level_breakdown[str(j)] = {"n": w["n_coarse"] << j, "us_per_pass": us,
+                                   "kernel": "line sweep" if by_lines[j] else pass_kernels[j],
                                    "passes_per_vcycle": passes, "ms_per_vcycle": us * passes / 1e3}
 
     # --- companions: FP64 and BF16-inverse V-cycles, time to 1e-8 ----------------
@@ -693,8 +732,8 @@ def main():
                 "gpu_launches": int(launches),
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                              "frac": achieved / hbm,
-                             "traffic": LINE_SWEEP_DRAM_BYTES.get(WORKLOAD),
-                             "kernel": "k_line_sweep<%d,%d,float,float> (finest level)" % (w["d"], w["degree"]),
+                             "traffic": traffic,
+                             "kernel": "%s<%d,%d,float,float> (finest level)" % (kernel, w["d"], w["degree"]),
                              "peak_kind": peak_kind, "avg_launch_ms": avg_launch_ms,
                              "bytes_per_launch": per_launch_bytes, "isolated_launch_ms": isolated_launch_ms,
                              "timing": f"two symmetric steps ({run_passes} passes in {len(runs)} launches) replayed as a "

@@ -86,6 +86,42 @@ def test_traffic_figures_are_the_committed_captures():
         assert abs(t / 1e6 - float(m.group(1))) < 0.006
 
 
+def test_line_sweep_launches_and_bytes():
+    """Launches of two symmetric steps and the bytes of the finest level's launches of
+    the default workload, by hand: 85 lines of 255 vertices a class, 7,225 patches a
+    colour; on each line 4 rows of 511 interior x nodes, 3 of 512 and 4 of 512 pressure
+    nodes.  A repeated colour of a five-pass launch streams no inverses again."""
+    runs = bench.smoothing_runs(2, True)
+    assert [len(q) for q in runs] == [3, 3, 5, 3, 5, 3, 5, 3, 3] and sum(runs, [])[:12] == [0, 1, 2, 3, 4, 5, 6, 7, 8, 7, 6, 5]
+    assert [len(q) for q in bench.smoothing_runs(2, False)] == [1] * 33
+    assert all(len({c // 3 for c in q}) == 1 for q in bench.smoothing_runs(3, True))
+    by_hand = 3 * 7225 * 1600 * 4 + 3 * 85 * (4 * 511 + 3 * 512 + 4 * 512) * 4
+    for q in runs:
+        assert bench.line_sweep_bytes(q, 2, 1, 256, [7225] * 9, 40, 4, 4) == by_hand
+    # the average launch's captured traffic is at most 15 % above it (repeated colours miss the cache in part)
+    assert by_hand <= bench.LINE_SWEEP_DRAM_BYTES["channels_256"] <= 1.15 * by_hand
+    # 3-D RT_0, 4^3: one line of three vertices in class (1, 1); 4 u_x rows of 3 nodes, 2 x 2 rows of u_y and u_z, 4 of p
+    assert bench.line_sweep_bytes([12, 13, 14], 3, 0, 4, [1] * 27, 20, 4, 4) == 3 * 400 * 4 + 3 * (4 * 3 + 2 * 2 * 4 + 4 * 4) * 4
+
+
+def test_smoother_kind_from_the_launches():
+    """A step of line sweeps launches fewer kernels than it has colour passes."""
+    class Handle:
+        def __init__(self, dim, per_step):
+            self.dim, self.n, self.per_step = dim, 0, per_step
+
+        def launches(self):
+            return self.n
+
+        def smooth(self, level, x, b, steps):
+            self.n += self.per_step
+
+    assert bench.smooths_by_lines(Handle(2, 5 + 3), 3, None, None)
+    assert bench.smooths_by_lines(Handle(3, 17 + 3), 3, None, None)
+    assert not bench.smooths_by_lines(Handle(2, 17), 3, None, None)
+    assert not bench.smooths_by_lines(Handle(3, 53 + 3), 3, None, None)
+
+
 def test_reference_arm_prints_the_contract_line(monkeypatch, capsys):
     """bench.py --impl reference: one JSON line with the keys of the benchmark
     contract, the reference arm's own cpu_baseline and e2e objects, and the
