@@ -97,8 +97,10 @@ typedef struct {
                            that differ in the x digit of the colour are one
                            launch, a cluster of blocks per line of vertices (not
                            with the additive variant, boundary_patches, a block
-                           limit, nor degree 2 in FP64).  The other values, and
-                           these where line sweeps do not apply, take one
+                           limit, degree 2 in FP64, nor degree 1 in FP64 where
+                           a colour's patches, over the right-hand sides, are
+                           no more than the device's SMs).  The other values,
+                           and these where line sweeps do not apply, take one
                            launch per colour pass: 1: one warp per patch
                            (persistent), 2: one thread block per patch,
                            3: persistent thread blocks, one patch at a time,

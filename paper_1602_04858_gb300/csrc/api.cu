@@ -223,12 +223,13 @@ bool host_constrained(const HostLevel& L, int64_t g) {
 // Passes of one launch of a line sweep (linepass.cuh).
 constexpr int LINE_RUN = 5;
 
-// Whether smoothing on level j runs as line sweeps: not with the additive
-// variant, the boundary-vertex patches (which follow every colour) or a cap on
-// the grid (mg_set_block_limit caps the persistent colour passes).
-bool line_sweeps(const mg_handle* h, int j) {
+// Whether smoothing of nrhs vectors on level j runs as line sweeps (fewer vectors than
+// the handle's as its V-cycle does, since its colour passes are timed for that number):
+// not with the additive variant, the boundary-vertex patches (which follow every colour)
+// or a cap on the grid (mg_set_block_limit caps the persistent colour passes).
+bool line_sweeps(const mg_handle* h, int j, int nrhs) {
   const HostLevel& L = h->lv[j];
-  return L.line && h->additive == 0.0 && L.max_blocks == 0 && L.bnv == 0;
+  return L.line > 0 && std::max(nrhs, h->nrhs) >= L.line && h->additive == 0.0 && L.max_blocks == 0 && L.bnv == 0;
 }
 
 // `steps` smoothing steps on level j for nrhs vectors x, b (acc: a level
@@ -256,7 +257,7 @@ mg_status smooth_steps(mg_handle* h, int j, void* x, const void* b, void* acc, i
     }
     return MG_OK;
   }
-  if (line_sweeps(h, j)) {
+  if (line_sweeps(h, j, nrhs)) {
     // runs of passes whose colours differ in the x digit only: one launch each
     // (a launch that fails ends the call: a V-cycle captured without it would be replayed)
     int cross = -1, ns = 0, cx[LINE_RUN];
@@ -603,7 +604,7 @@ mg_status refine_in_cycle(mg_handle* h, int nrhs) {
   float best = 0.f;
   bool timed_once = false;
   for (int j = h->J; j > h->Ls && j >= 1; --j) {
-    if (line_sweeps(h, j)) continue;   // no colour passes of their own in the cycle
+    if (line_sweeps(h, j, nrhs)) continue;   // no colour passes of their own in the cycle
     const Pick& a = timed[j];
     const Pick& r = rule[j];
     const bool single = nrhs < 4;
@@ -813,8 +814,8 @@ static mg_status setup_internal(const mg_problem* p, void* cuda_stream, int nrhs
     L.sprec = (h->prec == P32B && j < J) ? P32 : h->prec;
     if (j == 0) continue;
     // the kernel choices left to the library smooth by line sweeps (line_sweeps)
-    L.line = (p->pass_kernel == 0 || p->pass_kernel == 4 || p->pass_kernel == 5) && p->additive == 0.0 &&
-             !p->boundary_patches && h->ops->line_fits(L, L.sprec);
+    const bool lines = p->pass_kernel == 0 || p->pass_kernel == 4 || p->pass_kernel == 5;
+    L.line = lines && p->additive == 0.0 && !p->boundary_patches ? h->ops->line_fits(L, L.sprec) : 0;
     const size_t sb = (L.sprec == P64) ? 8 : (L.sprec == P32 ? 4 : 2);
     {
       int64_t np = 0;
@@ -1057,7 +1058,7 @@ mg_status mg_time_passes(mg_handle* h, int level, int kernel, double* us_per_pas
   float ms = 0.f;
   int64_t np = 0;
   const mg_status st = time_smoothing(h, level, h->nrhs, 2, 5, &ms, &np);
-  if (line_sweeps(h, level)) {   // colour passes of the two steps, several to a launch
+  if (line_sweeps(h, level, h->nrhs)) {   // colour passes of the two steps, several to a launch
     np = 0;
     const int C = num_colours(h->d);
     for (int s = 0; s < 2; ++s)

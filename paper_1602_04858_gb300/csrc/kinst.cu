@@ -779,7 +779,19 @@ int line_fits(const HostLevel& h, int prec) {
   // RT_2 in FP64 keeps the colour passes: its product has no lanes to spare and
   // one team per SM (26.5 against 22.7 us per pass on 64^2, 12.4 against 7.6 on 32^2)
   if (prec == P64) {
-    if constexpr (K < 2) return line_fits_t<double, double>(h);
+    if constexpr (K < 2) {
+      if (!line_fits_t<double, double>(h)) return 0;
+      if (K == 0) return 1;
+      // RT_1 in FP64 where a colour has no more patches than there are SMs, over the
+      // right-hand sides: a block each has an SM's FP64 units to itself, a warp of a sweep
+      // a quarter of them.  Colour passes / line sweeps (us per pass), one right-hand
+      // side: 8^2 2.8 / 4.5, 16^2 2.9 / 4.8, 32^2 (121 patches) 4.2 / 4.7, 40^2 (169) 7.5 /
+      // 4.8; four: 16^2 (100) 3.3 / 4.8, 24^2 (256) 6.2 / 4.8; sixteen: 8^2 (144) 3.5 / 4.5,
+      // 12^2 (256) 5.8 / 4.6
+      int64_t most = 1;
+      for (int e = 0; e < D; ++e) most *= (h.n - 1 + 2) / 3;
+      return (int)(num_sms() / most) + 1;
+    }
     return 0;
   }
   if (prec == P32) return line_fits_t<float, float>(h);

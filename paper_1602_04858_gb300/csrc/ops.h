@@ -81,8 +81,9 @@ struct HostLevel {
                          // are resident)
   int cta_tpr;           // threads per patch row of the block-per-patch pass for single right-hand
                          // sides: 4, 2 or 8
-  int line;              // 1: smoothing runs as line sweeps (linepass.cuh), the passes of one class of
-                         // vertex lines per launch, instead of one launch per colour pass
+  int line;              // smoothing of this many right-hand sides or more runs as line sweeps
+                         // (linepass.cuh), the passes of one class of vertex lines per launch, instead
+                         // of one launch per colour pass (0: never)
   int rhs_group;         // right-hand sides sharing each S_v load in the colour passes: 4 (groups
                          // of four where the count allows) or 1 (every right-hand side on its own)
   // problems of one shape stored one after another (grouped batches): rhs_prob
@@ -127,7 +128,8 @@ struct DKOps {
   // x digit + 3 cross), x digits cx[0 .. ns), in one launch; the launch's status
   cudaError_t (*line_sweep)(const HostLevel&, int cross, int ns, const int* cx, int prec, void* x, const void* b,
                             int* err, int nrhs, cudaStream_t);
-  // whether the level's strips fit the line sweep's shared memory
+  // right-hand sides from which line sweeps smooth the level (0: never, also where its
+  // strips do not fit the shared memory)
   int (*line_fits)(const HostLevel&, int prec);
   // patch inverses of one colour into S (storage precision sprec); *fail set on a zero pivot
   void (*patch_setup)(const HostLevel&, int colour, int sprec, void* S, int* fail, cudaStream_t);

@@ -4,7 +4,8 @@ set on every device that a thread uses one after the other, whatever split it
 has worked out before; a launch that fails is reported by the call and never
 becomes a replayed V-cycle without it; every problem of a batch smooths as its
 own pass_kernel asks; and what the line sweeps launch does not depend on the
-timings of the colour passes.  The library's own objects are linked
+timings of the colour passes; and small levels of RT_1 in FP64 smooth by colour
+passes.  The library's own objects are linked
 against the stand-in and run in a process of their own.
 """
 import os
@@ -109,7 +110,7 @@ def test_line_sweeps_do_not_follow_colour_pass_timings(lib, tmp_path, k, precisi
 L.fake_timings_fall({fall})
 G = handle({precision!r}, {k}, nrhs={nrhs})
 g = ctypes.c_int()
-L.mg_level_rhs_group(G.h, 2, ctypes.byref(g))
+L.mg_level_rhs_group(G.h, 4, ctypes.byref(g))
 assert g.value == (1 if {fall} else 4), g.value
 r = np.zeros({nrhs} * G.ndof())
 at = launches(b'k_line_sweep'), launches(b'Li4ELi1EEE'), launches(b'Li1ELi1EEE')
@@ -121,4 +122,26 @@ if {fall}:
     assert open(path).read() == repr(now), now
 else:
     open(path, 'w').write(repr(now))
+""")
+
+
+def test_small_fp64_levels_of_rt1_smooth_by_colour_passes(lib):
+    """152 SMs: a colour of 32^2 has at most 11^2 patches, one right-hand side stays
+    below, two do not; 40^2 has 13^2.  FP32 and RT_0 take line sweeps on every level,
+    and one vector on a handle of two goes as the handle's V-cycle does."""
+    run(lib, """
+def swept(n0, levels, nrhs, **kw):
+    G = handle(n0=n0, levels=levels, nrhs=nrhs, **kw)
+    r = np.zeros(nrhs * G.ndof())
+    at = launches(b'k_line_sweep')
+    G.vcycle(r, np.zeros_like(r))
+    v = launches(b'k_line_sweep') - at
+    at = launches(b'k_line_sweep')
+    G.smooth(levels - 1, np.zeros(G.ndof()), np.zeros(G.ndof()))
+    return v > 0, launches(b'k_line_sweep') - at > 0
+assert swept(4, 4, 1, precision='fp64') == (False, False)
+assert swept(4, 4, 2, precision='fp64') == (True, True)
+assert swept(5, 4, 1, precision='fp64') == (True, True)
+assert swept(4, 2, 1, precision='fp64', k=0) == (True, True)
+assert swept(4, 2, 1, precision='fp32') == (True, True)
 """)
