@@ -746,11 +746,11 @@ cudaError_t line_sweep_t(const HostLevel& h, int cross, int ns, const int* cx, v
   // (the colour passes' timed grouping is that of other kernels).  Small levels are
   // faster on their own (16^2 RT_1, 4 right-hand sides: 1.37 against 1.99 us per pass,
   // FP64 4.8 against 17), large ones in groups (128^2: 4.8 against 9.3).  The estimate
-  // flatters groups in FP64 and, less, from RT_1 on, and single vectors with BF16
-  // inverses; with these factors its choice takes 1 % longer than the faster one on
-  // average over 130 levels and numbers of right-hand sides, and nowhere over 10 %
+  // flatters groups in FP64 and, less, from RT_1 on, and in 3-D with BF16 inverses single
+  // vectors; with these factors its choice takes 1 % longer than the faster one on
+  // average over 138 levels and numbers of right-hand sides, and nowhere over 10 %
   // longer than groups.
-  constexpr double own = sizeof(T) == 8 ? 1.1 : (sizeof(TS) == 2 ? 0.95 : (K > 0 ? 1.06 : 1.0));
+  constexpr double own = sizeof(T) == 8 ? 1.1 : (K > 0 ? 1.06 : (D == 3 && sizeof(TS) == 2 ? 0.95 : 1.0));
   int g4 = (h.rhs_prob > 0 && h.rhs_prob % 4 != 0) ? 0 : nrhs / 4;
   if (g4 > 0 && line_split<T, TS, 1>(h, 4 * g4).t < own * line_split<T, TS, 4>(h, g4).t) g4 = 0;
   const int rest = nrhs - 4 * g4;
