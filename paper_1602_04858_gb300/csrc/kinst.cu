@@ -574,12 +574,14 @@ void line_attr() {
 // the device together (2,000).  How many clusters the device holds at once is asked
 // of the occupancy interface, since clusters do not cross the groups of SMs (of 3:
 // 46 with one block per SM, of 4: 36, of 6: 23, of 8: 15); a split that needs a
-// second wave for a few lines loses a third or more.  The constants were fitted to
+// second wave for a few lines loses a third or more, and so do clusters of five that by
+// those figures just fit (256^2 RT_1 with BF16 inverses 5 x 4: 9.8 us per pass, 6 x 3
+// 6.5): these count as needing the second wave.  The constants were fitted to
 // 4,000 measured splits of 43 levels (2-D RT_0 to RT_2, 3-D RT_0, FP32, FP64, BF16
 // inverses, 1 to 16 right-hand sides): the rule's splits take 2 % longer than the
 // best ones on average, 12 % at most.  Measured per pass (us): RT_1 256^2 3 x 6 7.2
 // (3 x 5 7.6, 6 x 7 8.2), FP64 3 x 6 49.3 (6 x 7 56.3); 128^2 6 x 7 2.74 (3 x 8
-// 2.99); 64^2 1.68 (1 x 11 above 2.2); 192^2 BF16 inverses 2 x 11 4.8 (6 x 4 4.3);
+// 2.99); 64^2 1.74 (1 x 11 above 2.6); 192^2 BF16 inverses 2 x 11 4.8 (6 x 4 4.3);
 // RT_0 128^2 1 x 11 1.31 (2 x 6 1.68); 3-D RT_0 64^3 1 x 11 4.5 (1 x 10 4.8), 32^3
 // 1 x 12 1.45 (1 x 11 of the other form 1.73).  The form of the kernel (LEAN) is
 // chosen the same way, by how many lines fit at once.
@@ -639,9 +641,11 @@ void line_split_form(int nx, int sms, int64_t lines, LineSplit& best) {
         }
         if (slots < 1) continue;
       }
-      // a last wave that is not full ends sooner
-      const double w = (double)lines / slots;
-      q.t = (run + (2 * lines > slots ? 2000.0 : 0.0)) * (w <= 1.0 ? 1.0 : 0.7 * std::ceil(w) + 0.3 * w);
+      // a last wave that is not full ends sooner; clusters of five that just fit the device
+      // do not all come up at once
+      double w = (double)lines / slots;
+      if (cl == 5 && w > 0.9 && w <= 1.0) w = 1.1;
+      q.t = (run + (2.0 * w > 1.0 ? 2000.0 : 0.0)) * (w <= 1.0 ? 1.0 : 0.7 * std::ceil(w) + 0.3 * w);
       if (best.cl == 0 || q.t < best.t || (q.t == best.t && q.cl == best.cl && MB == best.mb)) best = q;
     }
   }
