@@ -46,9 +46,9 @@
 // 1,500 clocks per pass).  What bounds it: on the finest level the inverses' bytes
 // (25 bytes per clock and SM), on coarse ones the chain of one patch update and
 // of the launch.  Measured per colour pass (GB300, passes back to back, us), colour
-// passes before and line sweeps: 2-D RT_1 FP32 256^2 10.7 -> 7.3, 128^2 3.8 ->
-// 2.7, 64^2 2.24 -> 1.69; FP64 256^2 58.6 -> 50.1; BF16 192^2 6.5 -> 4.4; RT_2 FP32
-// 128^2 23.3 -> 14.9; 3-D RT_0 FP32 64^3 7.5 -> 4.6; RT_0 512^2 5.6 -> 4.6.
+// passes and line sweeps: 2-D RT_1 FP32 256^2 10.6 and 7.2, 128^2 3.6 and 2.7, 64^2 2.23
+// and 1.74; FP64 256^2 58.6 and 49.3; BF16 192^2 6.5 and 4.8; RT_2 FP32 128^2 23.3 and
+// 14.9; 3-D RT_0 FP32 64^3 7.9 and 4.5; RT_0 512^2 5.6 and 4.1.
 #pragma once
 
 #include "passplan.cuh"
@@ -61,7 +61,7 @@ namespace mgd {
 // one lane, a pressure row GP (the second piece of one lane where GP = 0 or no
 // lane is left).  One warp per patch (RT_2: three) leaves least work outside the
 // slots; plans over 64 to 384 lanes, with a shorter chain of dependent work per
-// patch, were slower on every level measured (2-D RT_1 64^2: 2.24 against 1.69 us
+// patch, were slower on every level measured (2-D RT_1 64^2: 2.24 against 1.74 us
 // per pass; RT_2 128^2: 22.9 against 14.9).
 template <int D, int K> struct LinePlan;
 template <> struct LinePlan<2, 0> {   // 4 shared rows of at most 11 + 4 entries, 4 pressure rows of 4

@@ -161,15 +161,15 @@ struct DKOps {
   // bordered dense matrix of the coarsest level
   void (*coarse_assemble)(const HostLevel&, const int64_t* free_list, const int* g2l, int nf, double* M,
                           double* E, cudaStream_t);
+  // number of partial sums that residual_norm writes
+  int64_t (*residual_norm_count)(const HostLevel&);
   // FP64 r = b - A x (r may be null) and per-block partial sums of |r|^2;
   // returns the number of partials (blocks) written
-  int64_t (*residual_norm_count)(const HostLevel&);   // partial sums that residual_norm writes
   int64_t (*residual_norm)(const HostLevel&, const double* x, const double* b, double* r, double* partial,
                            cudaStream_t);
   // load vector of cellwise-constant f (D x ncell) and g (ncell, may be null), FP64
   void (*load_vector)(const HostLevel&, const double* f, const double* g, double* b, cudaStream_t);
-  // z[g] = r[g] on the constrained dofs (FP64), nvec vectors ndof apart
-  // z = X (of the handle's type) as FP64, on constrained rows r
+  // z = X (of the handle's type) as FP64, on constrained rows r; nvec vectors ndof apart
   void (*result)(const HostLevel&, int f32, const void* X, const double* r, double* z, int nvec, cudaStream_t);
 };
 
