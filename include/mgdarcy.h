@@ -241,10 +241,12 @@ mg_status mg_set_wait_limit(mg_handle* h, double seconds);
  * default), on the handle and its FP64 escalation hierarchy: leaves SMs to
  * concurrent work.  The kernels walk every patch of a colour whatever the
  * grid, and each patch's arithmetic does not depend on which block takes it,
- * so results are bit-identical for any cap (the test of one block walking a
+ * so results are bit-identical for any cap above 0, and where a pass_kernel
+ * of 1, 2 or 3 is asked for also without one (the test of one block walking a
  * whole colour relies on it).  With a cap the handle smooths by colour passes
- * even where it would take line sweeps (mg_problem.pass_kernel).  Re-captures the V-cycle graph on its next use;
- * synchronises the stream. */
+ * even where it would take line sweeps (mg_problem.pass_kernel), whose sums
+ * run in another order: capped and uncapped results then differ by rounding.
+ * Re-captures the V-cycle graph on its next use; synchronises the stream. */
 mg_status mg_set_block_limit(mg_handle* h, int blocks);
 
 /* Host buffer of `capacity` doubles that later mg_solve calls fill with the
